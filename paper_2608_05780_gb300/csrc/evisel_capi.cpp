@@ -690,6 +690,7 @@ int evisel_evidence_reduce(const evisel_ws* ws_c, float* tok, float* frame, floa
     T.tok = tok;
     T.frame = frame;
     T.status = ws->status;
+    for (const VideoInfo& v : P.videos) T.max_text = std::max<int>(T.max_text, v.n_text);
     T.n_chunks = static_cast<int>(P.chunks.size());
     T.n_tok = P.n_tok;
     T.hq = ws->hq;

@@ -177,8 +177,8 @@ struct CrossFrameLaunch {
   int* status;                      // device status word (a timed-out wait records EVISEL_ETIMEOUT)
 };
 
-// Text-row evidence by recompute (no logit spill): one CTA per (128 visual
-// keys, KV group).
+// Text-row evidence by recompute (no logit spill): units of (128 visual keys,
+// KV group, part of the group's heads).
 struct TextEvidenceLaunch {
   CUtensorMap tm_q, tm_k;           // 3-D maps {d, heads, tokens}, box {64, 1, 128}, 128B swizzle
   const EvChunk* chunks;
@@ -187,6 +187,8 @@ struct TextEvidenceLaunch {
   float* tok;                       // [hq, total_vis]
   float* frame;                     // [hq, total_frames]
   int* status;
+  int max_text;                     // most text rows of a video
+  int head_split, text_cols;        // parts of a KV group's heads, text rows per step (set by the launcher)
   int n_chunks, n_tok, hq, hkv, head_dim, tokens_per_frame, total_vis, total_frames;
   float scale_log2;
   int accumulate;
@@ -282,6 +284,21 @@ inline cudaError_t raise_smem_limit(PerDeviceAttr& once, const void* kern, int b
   e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
   if (e == cudaSuccess && bit) once.done.fetch_or(bit, std::memory_order_release);
   return e;
+}
+
+// SM count of the current device (cached per device; 0 if it cannot be read).
+inline int sm_count() {
+  static std::atomic<int> cached[64];
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0) return 0;
+  if (dev < 64) {
+    const int n = cached[dev].load(std::memory_order_relaxed);
+    if (n > 0) return n;
+  }
+  int n = 0;
+  if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
+  if (dev < 64) cached[dev].store(n, std::memory_order_relaxed);
+  return n;
 }
 
 // Bounded waits give up after this many nanoseconds of %globaltimer.

@@ -336,6 +336,8 @@ extern "C" int evisel_probe_evidence_noalloc(const evisel_probe_args* args, floa
       T.tok = tok;
       T.frame = frame;
       T.status = reinterpret_cast<int*>(base);
+      for (int b = 0; b < nb; ++b)
+        T.max_text = std::max(T.max_text, args->cu_seqlens_h[b + 1] - args->cu_seqlens_h[b] - args->n_vis_h[b]);
       T.n_chunks = static_cast<int>(c.chunks);
       T.n_tok = n_tok;
       T.hq = args->hq;

@@ -373,17 +373,6 @@ __global__ void __launch_bounds__(kThreads, 1) intra_frame_kernel(const __grid_c
   }
 }
 
-int sm_count() {
-  static int cached[64] = {};
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0) return 0;
-  if (dev < 64 && cached[dev] > 0) return cached[dev];
-  int n = 0;
-  if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
-  if (dev < 64) cached[dev] = n;
-  return n;
-}
-
 template <int D, int W>
 cudaError_t launch_dw(const IntraFrameLaunch& L, cudaStream_t stream) {
   using C = IfCfg<D>;
