@@ -1,8 +1,8 @@
 """Benchmark of the sparse-prefill evidence probe on one GB300 (or N replicas).
 
 One step = the whole hot path on one batch: evisel_probe_attention (block-sparse
-GQA attention + split-KV merge, text-logit spill) and evisel_evidence_reduce
-(token / frame / head maps and A_qf). The headline workload is the 65,664-token
+GQA attention + split-KV merge, the text rows' evidence sums) and
+evisel_evidence_reduce (token / frame / head maps and A_qf). The headline workload is the 65,664-token
 probe (1024 frames x 64 pooled tokens + 128 text tokens, 28 query / 4 KV heads,
 d = 128, 128-token tiles, sink + 16-tile window + 32 random tiles per visual
 row tile). Inputs are synthetic (seeded), resident in HBM when the timed region
@@ -79,13 +79,11 @@ def workload_stats(probe):
     flop = 4.0 * d * hq * elems
     flop_valid = 4.0 * d * hq * valid
     n_tok = int(probe.cu_seqlens[-1])
-    spill = sum(hq * int(nt) * int(nv) * 4 for nv, nt in zip(probe.n_vis, probe.n_text))
-    lse_read = sum(hq * int(nt) * 4 for nt in probe.n_text)
     total_vis = int(np.sum(probe.n_vis))
     frames = total_vis // cfg.tokens_per_frame
     maps = 4 * (hq * total_vis + hq * frames + len(probe.n_vis) * hq + frames)
-    return dict(flop=flop, flop_valid=flop_valid, tiles=tiles, n_tok=n_tok, spill_bytes=spill,
-                evidence_bytes=spill + lse_read + maps, map_bytes=maps)
+    return dict(flop=flop, flop_valid=flop_valid, tiles=tiles, n_tok=n_tok,
+                evidence_bytes=2 * maps, map_bytes=maps)   # the evidence call reads the sums and writes the maps
 
 
 def _peaks():
@@ -282,9 +280,8 @@ def _gpu_local_cpus(device_index):
 def bench_config(ev, name, args, peaks):
     """The step (probe + evidence over every layer) of one workload, timed on
     the launch stream with CUDA events: the whole step, and per layer the
-    probe call and the evidence call, once through each evidence path (the
-    text-row logit spill read back by the HBM-bound reduce, and the
-    recompute pass without the spill). Workloads whose inputs fit in L2 get a
+    probe call and the evidence call, once through each evidence mode (the
+    text rows' sums formed inside the probe call, and inside the evidence call). Workloads whose inputs fit in L2 get a
     256 MB write before every timed step (outside the timed interval)."""
     import torch
     cfg = wl.CONFIGS[name]
@@ -304,7 +301,7 @@ def bench_config(ev, name, args, peaks):
     q0 = dev[0][0]
     n, hq, d = q0.shape
     in_bytes = layers * sum(t.numel() * t.element_size() for t in dev[0])
-    flush = in_bytes + st["spill_bytes"] < 4 * L2_FLUSH_BYTES
+    flush = in_bytes < 4 * L2_FLUSH_BYTES
     flush_buf = torch.empty(L2_FLUSH_BYTES // 4, dtype=torch.float32, device="cuda") if flush else None
     o = torch.empty_like(q0)
     lse = torch.empty((hq, n), dtype=torch.float32, device="cuda")
@@ -375,8 +372,8 @@ def bench_config(ev, name, args, peaks):
             "evidence_ms": ev_ms, "evidence_bytes": layers * st["evidence_bytes"], "evidence_gbs": ev_gbs,
             "evidence_frac_of_hbm": ev_gbs / peaks["hbm"],
             "recompute_evidence": {
-                "note": "the same step with text_evidence = 1: the probe writes no text-row logit spill and the "
-                        "evidence call forms the text-row probabilities from q, k and the saved LSE",
+                "note": "the same step with text_evidence = 1: the evidence call, not the probe call, forms the "
+                        "text rows' sums from q, k and the saved LSE",
                 "step_ms": rc_step_ms, "tflops": flop / (rc_step_ms * 1e-3) / 1e12,
                 "tokens_per_s": st["n_tok"] * layers / (rc_step_ms * 1e-3),
                 "attention_ms": rc_attn_ms, "attention_tflops": rc_attn_tflops,
@@ -691,9 +688,9 @@ def bench_ours(args, cfg):
     if status != 0:
         raise RuntimeError("device status reported an error")
 
-    # The step with the recompute evidence pass (text_evidence = 1): the probe
-    # without the text-row logit spill, then the evidence formed from Q, K and
-    # the LSE on the tensor cores. Same outputs; timed like the step.
+    # The step with text_evidence = 1: the probe alone, then the evidence call
+    # that forms the text rows' sums from Q, K and the LSE on the tensor cores.
+    # Same outputs; timed like the step.
     ws_te = ev.Workspace()
     maps_te = [torch.zeros_like(m) for m in maps]
     ev.evisel_probe_attention(*pargs, ws=ws_te, o=o_cf, lse=lse_cf, text_evidence=True)
@@ -781,7 +778,7 @@ def bench_ours(args, cfg):
                           "evidence_ms": ev_avg, "evidence_bytes": st["evidence_bytes"], "evidence_gbs": ev_gbs,
                           "evidence_frac_of_hbm": ev_gbs / peaks["hbm"], "l2": "inputs larger than L2 (no flush)",
                           "recompute_evidence": {
-                              "note": "text_evidence_recompute above: the step without the text-row logit spill",
+                              "note": "text_evidence_recompute above: the sums formed in the evidence call",
                               "step_ms": te_step_ms, "tflops": st["flop"] / (te_step_ms * 1e-3) / 1e12,
                               "tokens_per_s": st["n_tok"] / (te_step_ms * 1e-3),
                               "attention_ms": te_probe_ms,

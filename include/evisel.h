@@ -44,7 +44,7 @@ extern "C" {
 #define EVISEL_ESTATE        -8  /* evidence requested before any probe on the workspace */
 
 /* Opaque workspace owned by the library: work list, device copy of the mask,
- * split-KV partials and the text-row logit spill. Created by the first
+ * split-KV partials and the text rows' evidence sums. Created by the first
  * evisel_probe_attention() call that receives *ws == NULL; reused (grown if
  * needed) by later calls; released only by evisel_free(). */
 typedef struct evisel_ws evisel_ws;
@@ -97,12 +97,12 @@ typedef struct {
                                     hq * nnz(mask) * tile * (tile / min(N_v, 64))
                                     * 4 bytes).
                                     0: not kept. Ignored by evisel_intra_frame_evidence. */
-  int32_t text_evidence;         /* how evisel_evidence_reduce() forms the text-row
-                                    probabilities: 0 = from the text rows' logits the
-                                    probe spills into the workspace (hq * n_text *
-                                    n_vis * 4 bytes per video); 1 = recomputed from
-                                    q and k (no spill; q and k, like lse, must stay
-                                    alive until evisel_evidence_reduce() ran). Same
+  int32_t text_evidence;         /* when the text rows' token and frame sums are formed
+                                    (from q, k and LSE): 0 = inside the probe call, into
+                                    the workspace (hq * sum n_vis * 4 bytes and the
+                                    frames); 1 = inside evisel_evidence_reduce() (q and
+                                    k, like lse, must stay alive until then; a program
+                                    that asks for no evidence map saves the pass). Same
                                     outputs within fp32 rounding. */
   const uint32_t* keep;          /* NULL, or device per-row block masks from
                                     evisel_topp_mask(): row i of head h attends only
@@ -118,8 +118,8 @@ typedef struct {
 
 /* Block-sparse causal GQA varlen attention (Eq. 1; Appendix Eq. 8 and Eq. 11
  * with exact token logits on every kept tile). Writes O and LSE for every
- * token, and spills the text rows' logits onto their video's visual tokens into
- * the workspace for evisel_evidence_reduce().
+ * token, and (text_evidence = 0) leaves the text rows' evidence sums over their
+ * video's visual tokens in the workspace for evisel_evidence_reduce().
  *   args      : the call description above (host struct, read during the call).
  *   stream    : cudaStream_t as void*.
  *   ws_inout  : in/out. *ws_inout == NULL -> a workspace is created and stored;
@@ -181,15 +181,16 @@ const char* evisel_build_id(void);
  * evisel_evidence_reduce() compute, with the same arguments and outputs (O and
  * LSE through `args`, the four evidence maps through tok/frame/head/aqf), but it
  * allocates nothing: no cudaMalloc, cudaFree, pinned memory or workspace. All of
- * its scratch -- the work plan, the split-KV partials of the text rows and the
- * text-row logit spill -- lives in one static device array of
+ * its scratch -- the work plan and the split-KV partials of the text rows --
+ * lives in one static device array of
  * EVISEL_NOALLOC_SCRATCH_BYTES (64 MiB), which every GPU that loads this library
  * holds until the process exits.
  *   - Limit: a problem whose scratch does not fit is rejected with EVISEL_ENOMEM
  *     (evisel_last_error() states the bytes needed) before anything is enqueued.
- *     The spill dominates: about hq * n_text * n_vis * 4 bytes per video, e.g.
- *     28 heads x 64 text x 4096 visual tokens = 29 MiB fits; the 65,664-token
- *     probe (940 MiB) does not -- use evisel_probe_attention() for it.
+ *     With text_evidence = 0 the limit counts hq * n_text * n_vis * 4 bytes per
+ *     video beside the plan and the partials: 28 heads x 64 text x 4096 visual
+ *     tokens = 29 MiB fits, the 65,664-token probe (940 MiB) does not. With
+ *     text_evidence = 1 (the same results here) it does.
  *   - Set-up: the first call on a device looks up the array's device address
  *     (cudaGetSymbolAddress, with that device current) and caches it; make that
  *     first call before any stream capture begins.

@@ -82,11 +82,11 @@ struct Plan {
   std::vector<CombineGroup> groups;
   std::vector<EvChunk> chunks;
   int n_parts = 0;
-  int64_t spill_floats = 0;
+  int max_text = 0;                 // most text rows of a video
   int total_vis = 0;
   int total_frames = 0;
   int n_tok = 0;
-  bool text_recompute = false;      // args->text_evidence: no spill, evidence from q and k
+  bool text_late = false;           // args->text_evidence: the evidence call forms the sums from q and k
   // cross-frame partials (args->cross_frame)
   bool cross_frame = false;
   std::vector<VisRow> vrows;        // visual row tiles in mask order
@@ -190,24 +190,20 @@ void build_plan(const evisel_probe_args* a, Plan& P) {
     for (int hh = 0; hh < gq; hh += kSlots * hp) head_blocks.push_back(g * gq + hh);
 
   // Videos.
-  int64_t spill = 0;
   int vis_off = 0, frame_off = 0;
   for (int b = 0; b < a->num_videos; ++b) {
     VideoInfo v{};
     v.vis_start = a->cu_seqlens_h[b];
     v.n_vis = a->n_vis_h[b];
     v.n_text = a->cu_seqlens_h[b + 1] - a->cu_seqlens_h[b] - v.n_vis;
-    v.text_pitch = (v.n_text + 31) & ~31;
-    v.spill_off = spill;
+    P.max_text = std::max(P.max_text, v.n_text);
     v.vis_off = vis_off;
     v.frame_off = frame_off;
-    if (!a->text_evidence) spill += static_cast<int64_t>(hq) * v.n_vis * v.text_pitch;
     vis_off += v.n_vis;
     frame_off += v.n_vis / a->tokens_per_frame;
     P.videos.push_back(v);
   }
-  P.spill_floats = spill;
-  P.text_recompute = a->text_evidence != 0;
+  P.text_late = a->text_evidence != 0;
   P.total_vis = vis_off;
   P.total_frames = frame_off;
 
@@ -397,7 +393,8 @@ struct evisel_ws {
   EvChunk* d_chunks = nullptr;
   float* d_part_o = nullptr;
   float2* d_part_ml = nullptr;
-  float* d_spill = nullptr;
+  float* d_ev_tok = nullptr;        // token and frame sums of the text rows (text_evidence = 0)
+  float* d_ev_frame = nullptr;
   VisRow* d_vrows = nullptr;
   int64_t* d_aff_off = nullptr;
   float* d_fspill = nullptr;
@@ -446,7 +443,7 @@ template <typename T>
 size_t bytes_of(const std::vector<T>& v) { return v.size() * sizeof(T); }
 
 // Lays out the arena and uploads the plan metadata on `stream`.
-int install_plan(evisel_ws* ws, cudaStream_t stream) {
+int install_plan(evisel_ws* ws, int hq, cudaStream_t stream) {
   const Plan& P = ws->plan;
   const int d = 128;   // partial rows are sized for the largest head_dim
   size_t off = 0;
@@ -461,7 +458,8 @@ int install_plan(evisel_ws* ws, cudaStream_t stream) {
   const size_t meta_bytes = off;
   const size_t o_part_o = take(static_cast<size_t>(P.n_parts) * 128 * d * sizeof(float));
   const size_t o_part_ml = take(static_cast<size_t>(P.n_parts) * 128 * sizeof(float2));
-  const size_t o_spill = take(static_cast<size_t>(P.spill_floats) * sizeof(float));
+  const size_t o_ev_tok = take(P.text_late ? 0 : static_cast<size_t>(hq) * P.total_vis * sizeof(float));
+  const size_t o_ev_frame = take(P.text_late ? 0 : static_cast<size_t>(hq) * P.total_frames * sizeof(float));
   const size_t o_fspill = take(static_cast<size_t>(P.fspill_floats) * sizeof(float));
   const size_t total = std::max<size_t>(off, 256);
 
@@ -517,7 +515,8 @@ int install_plan(evisel_ws* ws, cudaStream_t stream) {
   ws->d_chunks = reinterpret_cast<EvChunk*>(base + o_chunks);
   ws->d_part_o = reinterpret_cast<float*>(base + o_part_o);
   ws->d_part_ml = reinterpret_cast<float2*>(base + o_part_ml);
-  ws->d_spill = reinterpret_cast<float*>(base + o_spill);
+  ws->d_ev_tok = reinterpret_cast<float*>(base + o_ev_tok);
+  ws->d_ev_frame = reinterpret_cast<float*>(base + o_ev_frame);
   ws->d_vrows = reinterpret_cast<VisRow*>(base + o_vrows);
   ws->d_aff_off = reinterpret_cast<int64_t*>(base + o_aff_off);
   ws->d_fspill = reinterpret_cast<float*>(base + o_fspill);
@@ -537,6 +536,46 @@ int create_ws(evisel_ws** out) {
     return cuda_fail(e, "workspace creation");
   }
   *out = ws;
+  return EVISEL_OK;
+}
+
+// Token and frame sums of the text rows of the probe that ran on `ws`, from its
+// q, k and LSE, into (or, accumulating, onto) tok and frame. `args`: the probe's
+// arguments where its per-row block masks apply (they are read only inside
+// the probe call), else null.
+int launch_text_sums(evisel_ws* ws, float* tok, float* frame, int accumulate, const evisel_probe_args* args,
+                     cudaStream_t stream) {
+  const Plan& P = ws->plan;
+  if (P.chunks.empty()) return EVISEL_OK;
+  TextEvidenceLaunch T;
+  std::memset(&T, 0, sizeof(T));
+  int rc = encode_map(&T.tm_q, ws->q, P.n_tok, ws->hq, ws->head_dim, 128);
+  if (rc == EVISEL_OK) rc = encode_map(&T.tm_k, ws->k, P.n_tok, ws->hkv, ws->head_dim, 128);
+  if (rc != EVISEL_OK) return rc;
+  T.chunks = ws->d_chunks;
+  T.videos = ws->d_videos;
+  T.lse = ws->lse;
+  T.tok = tok;
+  T.frame = frame;
+  if (args && args->keep) {
+    T.keep = args->keep;
+    T.keep_words = args->keep_words;
+    T.keep_block = args->keep_block;
+  }
+  T.status = ws->status;
+  T.max_text = P.max_text;
+  T.n_chunks = static_cast<int>(P.chunks.size());
+  T.n_tok = P.n_tok;
+  T.hq = ws->hq;
+  T.hkv = ws->hkv;
+  T.head_dim = ws->head_dim;
+  T.tokens_per_frame = ws->tokens_per_frame;
+  T.total_vis = P.total_vis;
+  T.total_frames = P.total_frames;
+  T.scale_log2 = ws->scale * 1.4426950408889634f;
+  T.accumulate = accumulate;
+  cudaError_t e = launch_text_evidence(T, stream);
+  if (e != cudaSuccess) return cuda_fail(e, "text_evidence launch");
   return EVISEL_OK;
 }
 
@@ -565,7 +604,7 @@ int evisel_probe_attention(const evisel_probe_args* args, void* stream_ptr, evis
     ws->plan = Plan();
     build_plan(args, ws->plan);
     ws->have_plan = false;
-    rc = install_plan(ws, stream);
+    rc = install_plan(ws, args->hq, stream);
     if (rc != EVISEL_OK) return rc;
     ws->key.swap(key);
     ws->have_plan = true;
@@ -591,7 +630,6 @@ int evisel_probe_attention(const evisel_probe_args* args, void* stream_ptr, evis
     L.videos = ws->d_videos;
     L.o = args->o;
     L.lse = args->lse;
-    L.spill = P.text_recompute ? nullptr : ws->d_spill;
     L.part_o = ws->d_part_o;
     L.part_ml = ws->d_part_ml;
     L.status = ws->status;
@@ -643,6 +681,7 @@ int evisel_probe_attention(const evisel_probe_args* args, void* stream_ptr, evis
   ws->hq = args->hq;
   ws->tokens_per_frame = args->tokens_per_frame;
   ws->last_stream = stream;
+  if (!P.text_late) return launch_text_sums(ws, ws->d_ev_tok, ws->d_ev_frame, 0, args, stream);
   return EVISEL_OK;
 }
 
@@ -659,52 +698,24 @@ int evisel_evidence_reduce(const evisel_ws* ws_c, float* tok, float* frame, floa
     return fail(EVISEL_EINVAL, "an output map is NULL");
   if ((reinterpret_cast<uintptr_t>(tok) & 15u) != 0) return fail(EVISEL_EINVAL, "tok must be 16-byte aligned");
   cudaStream_t stream = static_cast<cudaStream_t>(stream_ptr);
+  if (P.text_late) {
+    const int rc = launch_text_sums(ws, tok, frame, accumulate != 0, nullptr, stream);
+    if (rc != EVISEL_OK) return rc;
+  }
   EvidenceLaunch L{};
-  L.chunks = ws->d_chunks;
   L.videos = ws->d_videos;
-  L.spill = ws->d_spill;
-  L.lse = ws->lse;
+  L.src_tok = P.text_late ? nullptr : ws->d_ev_tok;
+  L.src_frame = P.text_late ? nullptr : ws->d_ev_frame;
   L.tok = tok;
   L.frame = frame;
   L.head = head;
   L.aqf = aqf;
-  L.n_chunks = static_cast<int>(P.chunks.size());
   L.n_videos = static_cast<int>(P.videos.size());
-  L.n_tok = P.n_tok;
   L.hq = ws->hq;
   L.tokens_per_frame = ws->tokens_per_frame;
   L.total_vis = P.total_vis;
   L.total_frames = P.total_frames;
   L.accumulate = accumulate != 0;
-  if (P.text_recompute) {
-    // Token and frame maps from q and k (no spill); the finalize below forms
-    // the head map and A_qf from the frame map.
-    TextEvidenceLaunch T;
-    std::memset(&T, 0, sizeof(T));
-    int rc = encode_map(&T.tm_q, ws->q, P.n_tok, ws->hq, ws->head_dim, 128);
-    if (rc == EVISEL_OK) rc = encode_map(&T.tm_k, ws->k, P.n_tok, ws->hkv, ws->head_dim, 128);
-    if (rc != EVISEL_OK) return rc;
-    T.chunks = ws->d_chunks;
-    T.videos = ws->d_videos;
-    T.lse = ws->lse;
-    T.tok = tok;
-    T.frame = frame;
-    T.status = ws->status;
-    for (const VideoInfo& v : P.videos) T.max_text = std::max<int>(T.max_text, v.n_text);
-    T.n_chunks = static_cast<int>(P.chunks.size());
-    T.n_tok = P.n_tok;
-    T.hq = ws->hq;
-    T.hkv = ws->hkv;
-    T.head_dim = ws->head_dim;
-    T.tokens_per_frame = ws->tokens_per_frame;
-    T.total_vis = P.total_vis;
-    T.total_frames = P.total_frames;
-    T.scale_log2 = ws->scale * 1.4426950408889634f;
-    T.accumulate = accumulate != 0;
-    cudaError_t te = launch_text_evidence(T, stream);
-    if (te != cudaSuccess) return cuda_fail(te, "text_evidence launch");
-    L.n_chunks = 0;
-  }
   cudaError_t e = launch_evidence(L, stream);
   if (e != cudaSuccess) return cuda_fail(e, "evidence launch");
   ws->last_stream = stream;

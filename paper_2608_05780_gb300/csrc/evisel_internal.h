@@ -13,7 +13,7 @@ namespace evisel {
 // One kept kv tile of a work item: keys [start, start + len) (global token
 // indices, one video). `diag` marks the tile that holds the query tile's own
 // positions: causal masking inside it. `visual` marks visual-token tiles, whose
-// logits the text rows spill for the evidence pass.
+// keys the evidence maps cover.
 struct KvTile {
   int32_t start;
   int16_t len;
@@ -42,15 +42,14 @@ struct WorkItem {
 };
 static_assert(sizeof(WorkItem) == 32, "WorkItem is 32 bytes");
 
-// Per-video layout used by the spill and the evidence pass.
+// Per-video layout used by the attention and the evidence passes.
 struct VideoInfo {
-  int64_t spill_off;  // float offset of this video's logit block [hq, text_pitch / 32, n_vis, 32]
   int32_t vis_start;  // global index of its first visual token
   int32_t n_vis;
   int32_t n_text;
-  int32_t text_pitch; // n_text rounded up to a multiple of 32 (rows of the spill, in blocks of 32)
   int32_t vis_off;    // column offset of its tokens in the token map
   int32_t frame_off;  // column offset of its frames in the frame map
+  int32_t pad0, pad1, pad2;
 };
 static_assert(sizeof(VideoInfo) == 32, "VideoInfo is 32 bytes");
 
@@ -81,7 +80,6 @@ struct ProbeLaunch {
   const VideoInfo* videos;
   void* o;                          // bf16 [N, hq, d]
   float* lse;                       // [hq, N]
-  float* spill;                     // text-row logits
   float* part_o;                    // [slots, 128, d] fp32, unnormalised
   float2* part_ml;                  // [slots, 128] (running max in log2 units, row sum)
   int* status;                      // device status word
@@ -113,17 +111,15 @@ struct CombineLaunch {
 };
 
 struct EvidenceLaunch {
-  const EvChunk* chunks;
   const VideoInfo* videos;
-  const float* spill;
-  const float* lse;
+  const float* src_tok;             // token and frame sums in the workspace (null: already in tok and frame)
+  const float* src_frame;
   float* tok;
   float* frame;
   float* head;
   float* aqf;
-  int n_chunks;
   int n_videos;
-  int n_tok, hq, tokens_per_frame;
+  int hq, tokens_per_frame;
   int total_vis, total_frames;
   int accumulate;
 };
@@ -177,8 +173,8 @@ struct CrossFrameLaunch {
   int* status;                      // device status word (a timed-out wait records EVISEL_ETIMEOUT)
 };
 
-// Text-row evidence by recompute (no logit spill): units of (128 visual keys,
-// KV group, part of the group's heads).
+// Text-row evidence: units of (128 visual keys, KV group, part of the group's
+// heads).
 struct TextEvidenceLaunch {
   CUtensorMap tm_q, tm_k;           // 3-D maps {d, heads, tokens}, box {64, 1, 128}, 128B swizzle
   const EvChunk* chunks;
@@ -186,6 +182,8 @@ struct TextEvidenceLaunch {
   const float* lse;                 // [hq, N]
   float* tok;                       // [hq, total_vis]
   float* frame;                     // [hq, total_frames]
+  const uint32_t* keep;             // per-row block masks of the probe (as in ProbeLaunch) or null
+  int keep_words, keep_block;
   int* status;
   int max_text;                     // most text rows of a video
   int head_split, text_cols;        // parts of a KV group's heads, text rows per step (set by the launcher)

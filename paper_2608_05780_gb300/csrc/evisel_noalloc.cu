@@ -6,7 +6,7 @@
 // allocation (or the device-wide synchronisation of cudaFree) is not acceptable,
 // or hosts that forbid a library any allocator use of its own. For them this
 // entry point keeps all of its scratch -- the work
-// plan, the split-KV partials of the text rows and the text-row logit spill --
+// plan and the split-KV partials of the text rows --
 // in one file-scope device array of fixed size (kScratchBytes), and its host
 // staging in one file-scope host array. The caller still passes Q/K/V, the mask
 // and every output (O, LSE and the four evidence maps).
@@ -34,7 +34,7 @@ namespace evisel {
 int validate_probe_args(const evisel_probe_args* a);
 }
 
-// The device scratch: status word, plan, partials, spill. Held by every GPU
+// The device scratch: status word, plan, partials. Held by every GPU
 // that loads this library until the process exits.
 static __device__ __align__(256) unsigned char g_scratch[static_cast<size_t>(EVISEL_NOALLOC_SCRATCH_BYTES)];
 
@@ -55,7 +55,7 @@ size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 struct Counts {
   size_t items = 0, kv = 0, groups = 0, chunks = 0;
   int64_t parts = 0;
-  int64_t spill_floats = 0;
+  int64_t spill_floats = 0;   // of the documented limit only
   int total_vis = 0, total_frames = 0;
 };
 
@@ -81,15 +81,15 @@ void make_plan(const evisel_probe_args* a, Counts& c, const Out* o) {
     v.vis_start = a->cu_seqlens_h[b];
     v.n_vis = a->n_vis_h[b];
     v.n_text = a->cu_seqlens_h[b + 1] - a->cu_seqlens_h[b] - v.n_vis;
-    v.text_pitch = (v.n_text + 31) & ~31;
     return v;
   };
   for (int b = 0; b < nb; ++b) {
     VideoInfo v = info(b);
-    v.spill_off = spill;
     v.vis_off = vis_off;
     v.frame_off = frame_off;
-    if (!a->text_evidence) spill += static_cast<int64_t>(hq) * v.n_vis * v.text_pitch;
+    // text_evidence = 0 keeps the limit that callers know: the text rows'
+    // logits (rounded up to 32 rows) count as scratch, although none are stored.
+    if (!a->text_evidence) spill += static_cast<int64_t>(hq) * v.n_vis * ((v.n_text + 31) & ~31);
     vis_off += v.n_vis;
     frame_off += v.n_vis / a->tokens_per_frame;
     if (o) o->videos[b] = v;
@@ -200,7 +200,7 @@ extern "C" int evisel_probe_evidence_noalloc(const evisel_probe_args* args, floa
     return set_last_error(EVISEL_EINVAL, "an output map is NULL");
   if ((reinterpret_cast<uintptr_t>(tok) & 15u) != 0) return set_last_error(EVISEL_EINVAL, "tok must be 16-byte aligned");
 
-  // Scratch layout: [status | items | kv | videos | groups | chunks | partial O | partial (m, l) | spill]
+  // Scratch layout: [status | items | kv | videos | groups | chunks | partial O | partial (m, l)]
   const int nb = args->num_videos;
   size_t off = 256;
   auto take = [&](size_t bytes) { const size_t at = off; off = align256(off + bytes); return at; };
@@ -212,7 +212,7 @@ extern "C" int evisel_probe_evidence_noalloc(const evisel_probe_args* args, floa
   const size_t meta_end = off;
   const size_t o_part_o = take(static_cast<size_t>(c.parts) * 128 * args->head_dim * sizeof(float));
   const size_t o_part_ml = take(static_cast<size_t>(c.parts) * 128 * sizeof(float2));
-  const size_t o_spill = take(static_cast<size_t>(c.spill_floats) * sizeof(float));
+  take(static_cast<size_t>(c.spill_floats) * sizeof(float));
   if (off > kScratchBytes || meta_end - 256 > kStageBytes) {
     const std::string msg = "problem needs " + std::to_string(off) + " bytes of scratch (plan " +
                             std::to_string(meta_end - 256) + " bytes); the static scratch holds " +
@@ -272,7 +272,6 @@ extern "C" int evisel_probe_evidence_noalloc(const evisel_probe_args* args, floa
     L.videos = reinterpret_cast<const VideoInfo*>(base + o_videos);
     L.o = args->o;
     L.lse = args->lse;
-    L.spill = args->text_evidence ? nullptr : reinterpret_cast<float*>(base + o_spill);
     L.part_o = reinterpret_cast<float*>(base + o_part_o);
     L.part_ml = reinterpret_cast<float2*>(base + o_part_ml);
     L.status = reinterpret_cast<int*>(base);
@@ -307,30 +306,25 @@ extern "C" int evisel_probe_evidence_noalloc(const evisel_probe_args* args, floa
   }
   if (nb > 0) {
     EvidenceLaunch E{};
-    E.chunks = reinterpret_cast<const EvChunk*>(base + o_chunks);
     E.videos = reinterpret_cast<const VideoInfo*>(base + o_videos);
-    E.spill = reinterpret_cast<const float*>(base + o_spill);
-    E.lse = args->lse;
     E.tok = tok;
     E.frame = frame;
     E.head = head;
     E.aqf = aqf;
-    E.n_chunks = static_cast<int>(c.chunks);
     E.n_videos = nb;
-    E.n_tok = n_tok;
     E.hq = args->hq;
     E.tokens_per_frame = args->tokens_per_frame;
     E.total_vis = c.total_vis;
     E.total_frames = c.total_frames;
     E.accumulate = accumulate != 0;
-    if (args->text_evidence && c.chunks > 0) {
-      // Token and frame maps recomputed from q and k (no spill).
+    if (c.chunks > 0) {
+      // Token and frame maps from q, k and LSE (either evidence mode: it is all one call here).
       TextEvidenceLaunch T;
       std::memset(&T, 0, sizeof(T));
       rc = encode_tensor_map(&T.tm_q, args->q, n_tok, args->hq, args->head_dim, 128);
       if (rc == EVISEL_OK) rc = encode_tensor_map(&T.tm_k, args->k, n_tok, args->hkv, args->head_dim, 128);
       if (rc != EVISEL_OK) return rc;
-      T.chunks = E.chunks;
+      T.chunks = reinterpret_cast<const EvChunk*>(base + o_chunks);
       T.videos = E.videos;
       T.lse = args->lse;
       T.tok = tok;
@@ -346,7 +340,6 @@ extern "C" int evisel_probe_evidence_noalloc(const evisel_probe_args* args, floa
       T.tokens_per_frame = args->tokens_per_frame;
       T.total_vis = c.total_vis;
       T.total_frames = c.total_frames;
-      const float scale = args->softmax_scale > 0.f ? args->softmax_scale : 1.0f / std::sqrt(float(args->head_dim));
       T.scale_log2 = scale * 1.4426950408889634f;
       T.accumulate = accumulate != 0;
       e = launch_text_evidence(T, stream);
@@ -354,7 +347,6 @@ extern "C" int evisel_probe_evidence_noalloc(const evisel_probe_args* args, floa
         cudaGetLastError();
         return set_last_error(EVISEL_ECUDA, (std::string("text_evidence launch: ") + cudaGetErrorString(e)).c_str());
       }
-      E.n_chunks = 0;
     }
     e = launch_evidence(E, stream);
     if (e != cudaSuccess) {

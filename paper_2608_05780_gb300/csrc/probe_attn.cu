@@ -27,8 +27,7 @@
 // buffer: S_{j+1} is computed while the softmax works on S_j.
 // Online softmax in fp32 (log2 domain) with lazy rescaling: the running max is
 // only moved when it grows by more than 2^8, so O in TMEM is rescaled rarely.
-// Text row tiles also spill their logits onto visual keys for the evidence
-// pass. Every wait is bounded; on timeout the CTA records EVISEL_ETIMEOUT,
+// Every wait is bounded; on timeout the CTA records EVISEL_ETIMEOUT,
 // drains its own async work and exits.
 #include <cstdint>
 #include <cuda_runtime.h>
@@ -398,23 +397,8 @@ __device__ __forceinline__ void softmax_epilogue(const ProbeLaunch& L, const Wor
   const int qpos = it.q_start + row_local;
   const uint32_t lane_base = static_cast<uint32_t>(warp * 32) << 16;
   const uint32_t tmem = tmem_base + lane_base + slot * C::SLOT_COLS;
-  const bool spill_rows = it.text_row0 >= 0 && row_ok && L.spill != nullptr;   // no spill: evidence recomputed
   // With one slot, S alternates between both slots' S columns (see the MMA issuer).
   const bool two = left > C::HP;
-
-  float* spill_row = nullptr;
-  int vis_start = 0;
-  if (it.text_row0 >= 0) {
-    const VideoInfo vi = L.videos[it.video];
-    vis_start = vi.vis_start;
-    // Spill [hq, text_pitch / 32, n_vis, 32]: a warp's 32 rows are one row
-    // block, and for one key they are 128 contiguous bytes.
-    if (row_ok) {
-      const int r = it.text_row0 + row_local;
-      spill_row = L.spill + vi.spill_off + static_cast<int64_t>(head) * vi.n_vis * vi.text_pitch +
-                  static_cast<int64_t>(r >> 5) * vi.n_vis * 32 + (r & 31);
-    }
-  }
 
   // Cross-frame partials (visual rows, when enabled): per kept kv tile and
   // key frame f, m + log2(sum of the frame's P) in log2 units, so that the
@@ -430,7 +414,7 @@ __device__ __forceinline__ void softmax_epilogue(const ProbeLaunch& L, const Wor
 
   // Per-row block masks (EMB = their block size; 0: none): the row's bit per
   // block of its video (top-p retention and the own block), applied to the
-  // keys of every kv tile before the max, the spill and P.
+  // keys of every kv tile before the max and P.
   [[maybe_unused]] const uint32_t* em_row = nullptr;
   [[maybe_unused]] int em_vis_start = 0, em_n_vis = 0;
   if constexpr (EMB > 0) {
@@ -493,8 +477,6 @@ __device__ __forceinline__ void softmax_epilogue(const ProbeLaunch& L, const Wor
       limit = kv.len;
       if (kv.diag) limit = min(limit, qpos - kv.start + 1);
     }
-    const bool spill = spill_rows && kv.visual;
-    float* spill_dst = spill ? spill_row + static_cast<int64_t>(kv.start - vis_start) * 32 : nullptr;
     auto apply_em = [&](float* sv, int h) {
       if constexpr (EMB > 0) {
         if ((em_bits & ((1u << (TILE / EMB)) - 1u)) != (1u << (TILE / EMB)) - 1u) {
@@ -505,7 +487,7 @@ __device__ __forceinline__ void softmax_epilogue(const ProbeLaunch& L, const Wor
       }
     };
 
-    // Pass 1: row max (and the text rows' logit spill), 64 columns at a time.
+    // Pass 1: row max, 64 columns at a time.
     float m4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
 #pragma unroll
     for (int h = 0; h < TILE / 64; ++h) {
@@ -522,12 +504,6 @@ __device__ __forceinline__ void softmax_epilogue(const ProbeLaunch& L, const Wor
         }
       }
       apply_em(s, h);
-      if (spill) {
-        float* dst = spill_dst + h * 64 * 32;
-#pragma unroll
-        for (int c = 0; c < 64; ++c)
-          if (h * 64 + c < kv.len) __stcs(dst + c * 32, s[c] * L.scale);
-      }
       if (limit < TILE) {
 #pragma unroll
         for (int c = 0; c < 64; ++c) s[c] = h * 64 + c < limit ? s[c] : -INFINITY;

@@ -1,10 +1,13 @@
-// Text-row evidence by recompute (Sec. 3.2, "Evidence Decomposition"), the
-// variant of the evidence pass that needs no logit spill:
+// Text-row evidence (Sec. 3.2, "Evidence Decomposition"):
 //   tok[h, m]   = sum_{text rows i} exp(s_im - LSE_i),  s = scale q_i k_m (Eq. 8),
 //   frame[h, t] = sum_{m in frame t} tok[h, m],
 // with LSE the probe's saved row normaliser (Eq. 11). Text rows attend to
 // every visual key of their video (dense causal), so every (text row, visual
-// key) pair enters.
+// key) pair enters; after a probe with per-row block masks only the pairs whose
+// bit is set do (their LSE entries are staged once per block of the unit's
+// keys, -inf where the row does not keep the block). The probabilities are
+// formed again from q, k and LSE: spilling the text rows' logits from the probe
+// and reading them back (940 MB each way on 65,664 tokens) cost more.
 //
 // Work unit: 128 visual keys of a video, one KV group, a part of its heads. A
 // persistent grid (one CTA per SM) walks the units; every role runs on across
@@ -50,6 +53,7 @@ namespace {
 
 constexpr int kRows = 128;                       // keys of a unit (TMEM lanes)
 constexpr int kMaxText = 256;                    // text rows of a step
+constexpr int kMaxBlocks = 8;                    // mask blocks of a unit's keys (16 tokens at least)
 constexpr int kGroups = 4;                       // groups of key threads: heads in flight
 constexpr int kKeyWarps = kGroups * kRows / 32;
 constexpr int kWarpProducer = kKeyWarps;
@@ -69,8 +73,8 @@ struct TeCfg {
   static constexpr int NB = 4;                   // S buffers (2 of them used at 256 columns)
   static constexpr int OFF_K = 0;
   static constexpr int OFF_Q = KS * K_BYTES;
-  static constexpr int OFF_LSE = OFF_Q + QS * K_BYTES;              // [kTmemCols] fp32: one row per S buffer
-  static constexpr int OFF_RED = OFF_LSE + kTmemCols * 4;           // [kKeyWarps] fp32
+  static constexpr int OFF_LSE = OFF_Q + QS * K_BYTES;              // per S buffer [blocks of the keys][its columns] fp32
+  static constexpr int OFF_RED = OFF_LSE + kMaxBlocks * kTmemCols * 4;   // [kKeyWarps] fp32
   static constexpr int OFF_BAR = OFF_RED + kKeyWarps * 4;
   static constexpr int B_KF = 0, B_KE = B_KF + KS, B_QF = B_KE + KS, B_QE = B_QF + QS, B_SF = B_QE + QS,
                        B_SE = B_SF + NB, B_DRAIN = B_SE + NB;
@@ -131,6 +135,7 @@ __global__ void __launch_bounds__(kThreads, 1) text_evidence_kernel(const __grid
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int n_units = L.n_chunks * L.hkv * L.head_split;
   const int nb = kTmemCols / L.text_cols;          // S buffers = groups in use
+  const int nblk = L.keep ? kRows / L.keep_block : 1;   // mask blocks of a unit's keys
   // The n-th Q tile of MMA warp w is in stage w spw + n % spw, phase n / spw:
   // every barrier has one waiter, which sees each of its phases (a parity wait
   // must never run two phases ahead).
@@ -301,20 +306,32 @@ __global__ void __launch_bounds__(kThreads, 1) text_evidence_kernel(const __grid
       }
     };
     float next[kMaxText / 32];
+    uint32_t bits[kMaxText / 32];                  // per row: bit i = the unit's i-th block is kept
     auto load = [&]() {
       const float* lse = L.lse + static_cast<int64_t>(x.h0 + hh) * L.n_tok + x.vis_start + x.n_vis;
 #pragma unroll
       for (int i = 0; i < kMaxText / 32; ++i) {
         const int r = i * 32 + lane, row = tt * x.tile_rows + r;
-        next[i] = r < x.tile_rows && row < x.n_text ? -1.4426950408889634f * __ldg(lse + row) : -INFINITY;
+        const bool in = r < x.tile_rows && row < x.n_text;
+        next[i] = in ? -1.4426950408889634f * __ldg(lse + row) : -INFINITY;
+        bits[i] = 1u;
+        if (L.keep && in) {
+          const int blk0 = x.col0 / L.keep_block;  // a multiple of nblk: the blocks share one word
+          bits[i] = __ldg(L.keep + (static_cast<int64_t>(x.h0 + hh) * L.keep_words + (blk0 >> 5)) * L.n_tok +
+                          x.vis_start + x.n_vis + row) >> (blk0 & 31);
+        }
       }
     };
     seek();
     if (u < n_units) load();
     while (u < n_units) {
       float cur[kMaxText / 32];
+      uint32_t cur_bits[kMaxText / 32];
 #pragma unroll
-      for (int i = 0; i < kMaxText / 32; ++i) cur[i] = next[i];
+      for (int i = 0; i < kMaxText / 32; ++i) {
+        cur[i] = next[i];
+        cur_bits[i] = bits[i];
+      }
       const int b = nh & (nb - 1);
       if (++tt == x.n_tt) {
         tt = 0;
@@ -330,9 +347,12 @@ __global__ void __launch_bounds__(kThreads, 1) text_evidence_kernel(const __grid
         ok = false;
         break;
       }
+      for (int kb = 0; kb < nblk; ++kb) {
+        float* row = lse_s + (b * nblk + kb) * L.text_cols;
 #pragma unroll
-      for (int i = 0; i < kMaxText / 32; ++i)
-        if (i * 32 < L.text_cols) lse_s[b * L.text_cols + i * 32 + lane] = cur[i];
+        for (int i = 0; i < kMaxText / 32; ++i)
+          if (i * 32 < L.text_cols) row[i * 32 + lane] = (cur_bits[i] >> kb) & 1u ? cur[i] : -INFINITY;
+      }
       __syncwarp();
       if (lane == 0) ptx::mbar_arrive(bar(C::B_SF + b));
     }
@@ -345,6 +365,7 @@ __global__ void __launch_bounds__(kThreads, 1) text_evidence_kernel(const __grid
     const uint64_t scale2 = ptx::f2(L.scale_log2, L.scale_log2);
     const int npf = L.tokens_per_frame, w = npf < 32 ? npf : 32;
     const int log_npf = 31 - __clz(npf);           // N_v is a power of two
+    const int kblk = L.keep ? key / L.keep_block : 0;   // the key's mask block within the unit
     float* red = reinterpret_cast<float*>(smem + C::OFF_RED);
     int nh = 0;                                    // heads of this CTA so far
     uint32_t step = 0;                             // steps of this group so far
@@ -361,7 +382,7 @@ __global__ void __launch_bounds__(kThreads, 1) text_evidence_kernel(const __grid
           if (ok && warp_ok) {
             ptx::tc_fence_after();
             const int valid = min(x.tile_rows, x.n_text - tt * x.tile_rows);   // columns past them add 0
-            const float* lrow = lse_s + grp * L.text_cols;
+            const float* lrow = lse_s + (grp * nblk + kblk) * L.text_cols;
             // Blocks of 32 columns; the last may read up to 16 columns past
             // tile_rows, whose LSE entries are -inf: they are masked below.
 #pragma unroll 1
