@@ -8,11 +8,12 @@
 // slots use every K/V tile the CTA loads, and each slot's softmax runs while
 // the tensor core works on the other slot.
 //
-// Warp roles (352 threads):
+// Warp roles (352 threads; 384 for 128-token tiles, where the softmax warpgroups
+// take registers over from the third one):
 //   warps 0-3  softmax + epilogue of slot 0, one thread per query row (TMEM lane)
 //   warps 4-7  softmax + epilogue of slot 1
 //   warp 8     block set-up (mbarriers) and the loads of Q (both slots) and
-//              K_0, before the block-wide barrier; then K_j into an NS-deep ring
+//              K_0, before the block-wide barrier; then K_j into a 3-deep ring
 //   warp 10    TMA: V_j into an NS-deep ring (apart from K, so that K tiles
 //              run ahead of the V waits)
 //   warp 9     MMA issuer; the warp walks the tiles together and one elected
@@ -25,6 +26,15 @@
 // execute in issue order. An item with one slot (the last heads of a KV group
 // with an odd head count) uses the idle slot's S columns as a second S
 // buffer: S_{j+1} is computed while the softmax works on S_j.
+// What bounds it (65,664 tokens, clocks per kv tile of a two-slot item): 2150 of
+// tensor pipe; the MMA warp's loop (issue 2140, which blocks while the pipe is
+// busy, and its waits) and each slot's chain (softmax 1215, MMAs 1050, hand-overs
+// 450) both come to about 2700, so that neither alone can be improved. A K stage
+// comes free one kv tile before it is needed again with two stages, about the
+// latency of the load under load: the third one took the probe call from 3617 to
+// 3515 us (8-video batch 3412 -> 3320, one layer of the 28-layer probe 255 -> 248);
+// one pass over S, with P formed before the tile's max is known (see the
+// softmax), to 3455 (3304, 246).
 // Online softmax in fp32 (log2 domain) with lazy rescaling: the running max is
 // only moved when it grows by more than 2^8, so O in TMEM is rescaled rarely.
 // Every wait is bounded; on timeout the CTA records EVISEL_ETIMEOUT,
@@ -39,11 +49,14 @@ namespace evisel {
 namespace {
 
 static_assert(kSlots == 2, "the kernel runs two slots per work item");
-constexpr int kThreads = 352;
+// 128-token tiles: three warpgroups that trade registers (warp 11 has no role).
+template <int TILE>
+constexpr int kThreads = TILE == 128 ? 384 : 352;
 constexpr int kWarpProducer = 8;   // Q, then the K ring
 constexpr int kWarpMma = 9;
 constexpr int kWarpVLoader = 10;   // the V ring
 constexpr int kRows = 128;
+constexpr int NK = 3;                  // stages of the K ring (the V ring has NS; shared memory holds no more)
 constexpr float kRescaleThreshold = 8.0f;   // log2 units
 constexpr float kLn2 = 0.69314718055994531f;
 
@@ -57,13 +70,13 @@ struct Cfg {
   static constexpr int KV_BYTES = TILE * D * 2;
   static constexpr int OFF_Q = 0;                        // two slots
   static constexpr int OFF_K = OFF_Q + 2 * Q_BYTES;
-  static constexpr int OFF_V = OFF_K + NS * KV_BYTES;
+  static constexpr int OFF_V = OFF_K + NK * KV_BYTES;
   static constexpr int OFF_BAR = OFF_V + NS * KV_BYTES;
   // barrier indices
   static constexpr int B_Q = 0;
-  static constexpr int B_KF = 1;             // NS: K tile landed
-  static constexpr int B_KE = B_KF + NS;     // NS: K tile consumed by both S MMAs
-  static constexpr int B_VF = B_KE + NS;     // NS: V tile landed
+  static constexpr int B_KF = 1;             // NK: K tile landed
+  static constexpr int B_KE = B_KF + NK;     // NK: K tile consumed by both S MMAs
+  static constexpr int B_VF = B_KE + NK;     // NS: V tile landed
   static constexpr int B_VE = B_VF + NS;     // NS: V tile consumed by both P.V MMAs
   static constexpr int B_SF = B_VE + NS;     // 2 (per slot): S_j computed
   static constexpr int B_PF = B_SF + 2;      // 2 (per slot): P_j written (128 arrivals)
@@ -95,6 +108,19 @@ __device__ __forceinline__ void record_failure(volatile int* abort_flag, int* st
 __device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
   const bool ok = ptx::mbar_wait(bar, parity, abort_flag, kWaitTimeoutNs);
   return __all_sync(0xffffffffu, ok);
+}
+
+struct Wait {
+  uint32_t bar, parity;
+};
+// Waits for `last` after two barriers that are usually over (their tests and the
+// wait issue back to back, with one vote).
+__device__ __forceinline__ bool warp_wait(Wait a, Wait b, Wait last, volatile int* abort_flag) {
+  const bool seen = static_cast<int>(ptx::mbar_test(a.bar, a.parity)) & static_cast<int>(ptx::mbar_test(b.bar, b.parity)) &
+                    static_cast<int>(ptx::mbar_try_wait(last.bar, last.parity));
+  if (__all_sync(0xffffffffu, seen)) return true;
+  return warp_wait(a.bar, a.parity, abort_flag) && warp_wait(b.bar, b.parity, abort_flag) &&
+         warp_wait(last.bar, last.parity, abort_flag);
 }
 
 // Heads of the item's KV group from its first head on.
@@ -165,11 +191,12 @@ __device__ __forceinline__ void producer(const ProbeLaunch& L, const WorkItem& i
   const int off = IS_V ? C::OFF_V : C::OFF_K;
   const int b_full = IS_V ? C::B_VF : C::B_KF;
   const int b_empty = IS_V ? C::B_VE : C::B_KE;
+  constexpr int R = IS_V ? NS : NK;              // ring stages
   const int first = (IS_V || n == 0) ? 0 : 1;   // K tile 0 went out with the set-up
   int issued = first;
   for (int j = first; j < n; ++j) {
-    const int s = j % NS;
-    const int u = j / NS;
+    const int s = j % R;
+    const int u = j / R;
     const int kv_start = __shfl_sync(0xffffffffu, L.kv[kv_begin + j].start, 0);
     if (u > 0 && !warp_wait(bar(b_empty + s), (u - 1) & 1, abort_flag)) {
       if ((threadIdx.x & 31) == leader) record_failure(abort_flag, L.status, kStatusTimeout);
@@ -191,9 +218,9 @@ __device__ __forceinline__ void producer(const ProbeLaunch& L, const WorkItem& i
     // when the CTA exits, whether or not another warp gave up.
     const volatile int never = 0;
     if (!IS_V) ptx::mbar_wait(bar(C::B_Q), 0, &never, kWaitTimeoutNs);
-    for (int s = 0; s < NS && s < issued; ++s) {
-      const int last = ((issued - 1 - s) / NS) * NS + s;
-      ptx::mbar_wait(bar(b_full + s), (last / NS) & 1, &never, kWaitTimeoutNs);
+    for (int s = 0; s < R && s < issued; ++s) {
+      const int last = ((issued - 1 - s) / R) * R + s;
+      ptx::mbar_wait(bar(b_full + s), (last / R) & 1, &never, kWaitTimeoutNs);
     }
   }
 }
@@ -228,14 +255,13 @@ __device__ __forceinline__ void mma_issuer(const ProbeLaunch& L, const WorkItem&
   const uint64_t dq0 = ptx::sdesc_sw128(sbase + C::OFF_Q, 16, 1024);
   const uint64_t dq1 = ptx::sdesc_sw128(sbase + C::OFF_Q + C::Q_BYTES, 16, 1024);
   const uint64_t dk0 = ptx::sdesc_sw128(sbase + C::OFF_K, 16, 1024);
-  const uint64_t dk1 = ptx::sdesc_sw128(sbase + C::OFF_K + C::KV_BYTES, 16, 1024);
   const uint64_t dv0 = ptx::sdesc_sw128(sbase + C::OFF_V, C::KV_BLOCK, 1024);
   const uint64_t dv1 = ptx::sdesc_sw128(sbase + C::OFF_V + C::KV_BYTES, C::KV_BLOCK, 1024);
   static_assert(NS == 2, "two ring stages");
   // S[buf] = Q_slot K_j^T (buf: whose S columns receive it)
   auto mma_s = [&](int slot, int j, int buf) {
     const uint64_t qd = slot ? dq1 : dq0;
-    const uint64_t kd = (j & 1) ? dk1 : dk0;
+    const uint64_t kd = dk0 + static_cast<uint64_t>((j % NK) * C::KV_BYTES >> 4);
     const uint32_t d_tmem = tmem + buf * C::SLOT_COLS + C::COL_S;
 #pragma unroll
     for (int kk = 0; kk < D / 16; ++kk) {
@@ -274,13 +300,13 @@ __device__ __forceinline__ void mma_issuer(const ProbeLaunch& L, const WorkItem&
       ok = same_leader;
     }
     if (ok && n > 1) {
-      if (!warp_wait(bar(C::B_KF + 1 % NS), (1 / NS) & 1, abort_flag)) {
+      if (!warp_wait(bar(C::B_KF + 1), 0, abort_flag)) {
         ok = false;
       } else {
         if (elect()) {
           mma_s(0, 1, 1);
           ptx::mma_commit(bar(C::B_SF + 1));
-          ptx::mma_commit(bar(C::B_KE + 1 % NS));
+          ptx::mma_commit(bar(C::B_KE + 1));
         }
         __syncwarp();
         ok = same_leader;
@@ -289,11 +315,11 @@ __device__ __forceinline__ void mma_issuer(const ProbeLaunch& L, const WorkItem&
     for (int j = 0; ok && j < n; ++j) {
       const int b = j & 1;
       const int s = j % NS;
-      const int s2 = (j + 2) % NS;
+      const int s2 = (j + 2) % NK;
       const bool more = j + 2 < n;
-      if ((more && !warp_wait(bar(C::B_KF + s2), ((j + 2) / NS) & 1, abort_flag)) ||
-          !warp_wait(bar(C::B_VF + s), (j / NS) & 1, abort_flag) ||
-          !warp_wait(bar(C::B_PF + b), (j >> 1) & 1, abort_flag)) {
+      const Wait v{bar(C::B_VF + s), static_cast<uint32_t>(j / NS) & 1u};
+      const Wait kn = more ? Wait{bar(C::B_KF + s2), static_cast<uint32_t>((j + 2) / NK) & 1u} : v;
+      if (!warp_wait(v, kn, Wait{bar(C::B_PF + b), static_cast<uint32_t>(j >> 1) & 1u}, abort_flag)) {
         ok = false;
         break;
       }
@@ -327,12 +353,13 @@ __device__ __forceinline__ void mma_issuer(const ProbeLaunch& L, const WorkItem&
     }
     for (int j = 0; ok && j < n; ++j) {
       const int s = j % NS;
-      const int s1 = (j + 1) % NS;
+      const int s1 = (j + 1) % NK;
       const bool more = j + 1 < n;
-      // The K/V tiles landed long ago in steady state: test them before P0 so
-      // that P0's arrival starts P0.V and the next S0 at once.
-      if ((more && !warp_wait(bar(C::B_KF + s1), ((j + 1) / NS) & 1, abort_flag)) ||
-          !warp_wait(bar(C::B_VF + s), (j / NS) & 1, abort_flag) || !warp_wait(bar(C::B_PF), j & 1, abort_flag)) {
+      // The K/V tiles landed long ago in steady state: they are tested together
+      // with P0, whose arrival starts P0.V and the next S0 at once.
+      const Wait v{bar(C::B_VF + s), static_cast<uint32_t>(j / NS) & 1u};
+      const Wait kn = more ? Wait{bar(C::B_KF + s1), static_cast<uint32_t>((j + 1) / NK) & 1u} : v;
+      if (!warp_wait(v, kn, Wait{bar(C::B_PF), static_cast<uint32_t>(j) & 1u}, abort_flag)) {
         ok = false;
         break;
       }
@@ -453,6 +480,7 @@ __device__ __forceinline__ void softmax_epilogue(const ProbeLaunch& L, const Wor
     if (it.kv_count > 0) em_next = mask_word(kv_next);
   }
 
+  bool watch = true;          // warp-uniform: take this tile's max before its P
   for (int j = 0; j < it.kv_count; ++j) {
     KvTile kv;
     [[maybe_unused]] uint32_t em_bits = 0xffffffffu;
@@ -471,122 +499,60 @@ __device__ __forceinline__ void softmax_epilogue(const ProbeLaunch& L, const Wor
     const uint32_t bar_pf = bar(C::B_PF + b);
     if (!warp_wait(bar(C::B_SF + b), par, abort_flag)) { ok = false; break; }
     ptx::tc_fence_after();
-    // Keys past the tile's end (ragged tile) or above the diagonal are masked.
-    int limit = TILE;
-    if (kv.diag || kv.len < TILE) {
+    int limit = TILE;                        // keys from here on are masked:
+    if (kv.diag || kv.len < TILE) {          // past the tile's end (ragged tile) or above the diagonal
       limit = kv.len;
       if (kv.diag) limit = min(limit, qpos - kv.start + 1);
     }
-    auto apply_em = [&](float* sv, int h) {
+    // 64 columns of the row's S: masks, then max.
+    auto mask64 = [&](uint32_t (&r)[2][32], int h) {
       if constexpr (EMB > 0) {
         if ((em_bits & ((1u << (TILE / EMB)) - 1u)) != (1u << (TILE / EMB)) - 1u) {
 #pragma unroll
           for (int c = 0; c < 64; ++c)
-            if (!((em_bits >> ((h * 64 + c) / EMB)) & 1u)) sv[c] = -INFINITY;
+            if (!((em_bits >> ((h * 64 + c) / EMB)) & 1u)) r[c / 32][c % 32] = 0xff800000u;   // -inf
         }
       }
-    };
-
-    // Pass 1: row max, 64 columns at a time.
-    float m4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
-#pragma unroll
-    for (int h = 0; h < TILE / 64; ++h) {
-      float s[64];
-      {
-        uint32_t r0[32], r1[32];
-        ptx::tmem_ld32(tS + h * 64, r0);
-        ptx::tmem_ld32(tS + h * 64 + 32, r1);
-        ptx::tmem_wait_ld();
-#pragma unroll
-        for (int e = 0; e < 32; ++e) {
-          s[e] = __uint_as_float(r0[e]);
-          s[32 + e] = __uint_as_float(r1[e]);
-        }
-      }
-      apply_em(s, h);
       if (limit < TILE) {
 #pragma unroll
-        for (int c = 0; c < 64; ++c) s[c] = h * 64 + c < limit ? s[c] : -INFINITY;
+        for (int c = 0; c < 64; ++c)
+          if (h * 64 + c >= limit) r[c / 32][c % 32] = 0xff800000u;
       }
+    };
+    auto max64 = [&](const uint32_t (&r)[2][32], float (&m4)[4]) {
 #pragma unroll
       for (int c = 0; c < 64; c += 8) {
-        m4[0] = ptx::max3(m4[0], s[c], s[c + 1]);
-        m4[1] = ptx::max3(m4[1], s[c + 2], s[c + 3]);
-        m4[2] = ptx::max3(m4[2], s[c + 4], s[c + 5]);
-        m4[3] = ptx::max3(m4[3], s[c + 6], s[c + 7]);
-      }
-    }
-    const float mx = fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3]));
-    const float m_tile = mx * L.scale_log2;
-    const bool need = m_tile > m_used + kRescaleThreshold;
-    float alpha = 1.f;
-    if (need) {
-      alpha = ptx::ex2(m_used - m_tile);
-      l_sum *= alpha;
-      m_used = m_tile;
-    }
-    const float m_safe = (m_used == -INFINITY) ? 0.f : m_used;
-
-    // Lazy rescale of the O accumulator (only rows whose max moved by > 2^8).
-    // With two slots S_j was issued after P_{j-1}.V, so that MMA has
-    // completed; with one slot it is waited for (its V-empty barrier).
-    if (j > 0 && __any_sync(0xffffffffu, need)) {
-      if (!two && !warp_wait(bar(C::B_VE + (j - 1) % NS), ((j - 1) / NS) & 1, abort_flag)) {
-        ok = false;
-        break;
-      }
-      ptx::tc_fence_after();
 #pragma unroll
-      for (int c = 0; c < D / 32; ++c) {
-        uint32_t r[32];
-        ptx::tmem_ld32(tmem + C::COL_O + c * 32, r);
-        ptx::tmem_wait_ld();
-#pragma unroll
-        for (int e = 0; e < 32; ++e) r[e] = __float_as_uint(__uint_as_float(r[e]) * alpha);
-        ptx::tmem_st32(tmem + C::COL_O + c * 32, r);
+        for (int e = 0; e < 4; ++e)
+          m4[e] = ptx::max3(m4[e], __uint_as_float(r[c / 32][c % 32 + 2 * e]),
+                            __uint_as_float(r[c / 32][c % 32 + 2 * e + 1]));
       }
-    }
-
-    // Pass 2: P = 2^(s * scale * log2 e - m) in packed pairs, written as bf16
-    // over the first half of S (columns of a 64-wide chunk are read before
-    // the chunk's P is stored, and P of chunk h lands below chunk h + 1).
-    const uint64_t negm2 = ptx::f2(-m_safe, -m_safe);
-    uint64_t l2[4] = {0, 0, 0, 0};
-    [[maybe_unused]] float l_tile = 0.f;
+    };
+    auto load64 = [&](uint32_t (&r)[2][32], int h) {
+      ptx::tmem_ld32(tS + h * 64, r[0]);
+      ptx::tmem_ld32(tS + h * 64 + 32, r[1]);
+    };
     [[maybe_unused]] float* fs_tile = nullptr;
     if constexpr (FSW > 0) {
       if (fs_row) fs_tile = fs_row + static_cast<int64_t>(j) * (TILE / FSW) * TILE;
     }
+    uint64_t l2[4];
+    [[maybe_unused]] float l_tile;
+    float m_safe;
+    uint64_t negm2;
+    // P of 32 columns (q-th quarter of the tile): 2^(s * scale * log2 e - m) in
+    // packed pairs, as bf16 into pk.
+    auto p32 = [&](const uint32_t (&r)[32], int q, uint32_t (&pk)[32]) {
 #pragma unroll
-    for (int h = 0; h < TILE / 64; ++h) {
-      float s[64];
-      {
-        uint32_t r0[32], r1[32];
-        ptx::tmem_ld32(tS + h * 64, r0);
-        ptx::tmem_ld32(tS + h * 64 + 32, r1);
-        ptx::tmem_wait_ld();
-#pragma unroll
-        for (int e = 0; e < 32; ++e) {
-          s[e] = __uint_as_float(r0[e]);
-          s[32 + e] = __uint_as_float(r1[e]);
-        }
-      }
-      apply_em(s, h);
-      if (limit < TILE) {
-#pragma unroll
-        for (int c = 0; c < 64; ++c) s[c] = h * 64 + c < limit ? s[c] : -INFINITY;
-      }
-      uint32_t pk[32];
-#pragma unroll
-      for (int e = 0; e < 32; ++e) {
+      for (int e = 0; e < 16; ++e) {
         float x0, x1;
-        ptx::unf2(ptx::fma2(ptx::f2(s[2 * e], s[2 * e + 1]), scale2, negm2), x0, x1);
+        ptx::unf2(ptx::fma2(ptx::f2(__uint_as_float(r[2 * e]), __uint_as_float(r[2 * e + 1])), scale2, negm2), x0, x1);
         const float p0 = ptx::ex2(x0);
         const float p1 = ptx::ex2(x1);
         l2[e & 3] = ptx::add2(l2[e & 3], ptx::f2(p0, p1));
-        pk[e] = ptx::pack_bf16x2(p0, p1);
+        pk[(q & 1) * 16 + e] = ptx::pack_bf16x2(p0, p1);
         if constexpr (FSW > 0) {
-          if ((h * 64 + 2 * e + 2) % FSW == 0) {      // the last keys of span (h * 64 + 2e + 2) / FSW - 1
+          if ((q * 32 + 2 * e + 2) % FSW == 0) {      // the last keys of span (q * 32 + 2e + 2) / FSW - 1
             float a0, a1, b0, b1, c0, c1, d0, d1;
             ptx::unf2(l2[0], a0, a1);
             ptx::unf2(l2[1], b0, b1);
@@ -596,11 +562,89 @@ __device__ __forceinline__ void softmax_epilogue(const ProbeLaunch& L, const Wor
             l_tile += fsum;
             l2[0] = l2[1] = l2[2] = l2[3] = 0;
             if (fs_tile)
-              __stcs(fs_tile + ((h * 64 + 2 * e + 2) / FSW - 1) * TILE, fsum > 0.f ? m_safe + __log2f(fsum) : -INFINITY);
+              __stcs(fs_tile + ((q * 32 + 2 * e + 2) / FSW - 1) * TILE, fsum > 0.f ? m_safe + __log2f(fsum) : -INFINITY);
           }
         }
       }
-      ptx::tmem_st32(tS + h * 32, pk);
+    };
+    auto begin_p = [&]() {
+      m_safe = (m_used == -INFINITY) ? 0.f : m_used;
+      negm2 = ptx::f2(-m_safe, -m_safe);
+      l2[0] = l2[1] = l2[2] = l2[3] = 0;
+      l_tile = 0.f;
+    };
+
+    uint32_t ra[2][32], rb[2][32], pk[32];   // S: first and second half of the tile
+    bool max_first = TILE == 64 || watch;    // (a 64-key tile gains nothing from the early half)
+    if (!max_first) {
+      // The running max holds for nearly every tile: P of the first half is
+      // formed with it while the tile's max is taken, and stands if no row of
+      // the warp needs a larger one. The second half loads meanwhile.
+      begin_p();
+      float m4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+      load64(ra, 0);
+      ptx::tmem_wait_ld();
+      if constexpr (TILE == 128) load64(rb, 1);
+      mask64(ra, 0);
+      max64(ra, m4);
+      p32(ra[0], 0, pk);
+      if constexpr (TILE == 128) {
+        ptx::tmem_wait_ld();
+        mask64(rb, 1);
+        max64(rb, m4);
+      }
+      p32(ra[1], 1, pk);
+      const float m_tile = fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3])) * L.scale_log2;
+      max_first = __any_sync(0xffffffffu, m_tile > m_used + kRescaleThreshold);
+    }
+    if (max_first) {
+      // The first tile, a row whose max grew by more than 2^8, or the tile after
+      // such a one (maxima that move tend to move again): the max first, then
+      // the lazy rescale of the row sum and (not on the first tile) of the O
+      // accumulator. With two slots S_j was issued after P_{j-1}.V, so that
+      // MMA has completed; with one slot it is waited for (its V-empty barrier).
+      float m4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+      load64(ra, 0);
+      if constexpr (TILE == 128) load64(rb, 1);
+      ptx::tmem_wait_ld();
+      mask64(ra, 0);
+      max64(ra, m4);
+      if constexpr (TILE == 128) {
+        mask64(rb, 1);
+        max64(rb, m4);
+      }
+      const float m_tile = fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3])) * L.scale_log2;
+      const bool need = m_tile > m_used + kRescaleThreshold;
+      watch = __any_sync(0xffffffffu, need);
+      const float alpha = need ? ptx::ex2(m_used - m_tile) : 1.f;
+      l_sum *= alpha;
+      m_used = need ? m_tile : m_used;
+      if (watch && j > 0) {
+        if (!two && !warp_wait(bar(C::B_VE + (j - 1) % NS), ((j - 1) / NS) & 1, abort_flag)) {
+          ok = false;
+          break;
+        }
+        ptx::tc_fence_after();
+#pragma unroll 1
+        for (int c = 0; c < D / 16; ++c) {
+          uint32_t o[16];
+          ptx::tmem_ld16(tmem + C::COL_O + c * 16, o);
+          ptx::tmem_wait_ld();
+#pragma unroll
+          for (int e = 0; e < 16; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * alpha);
+          ptx::tmem_st16(tmem + C::COL_O + c * 16, o);
+        }
+      }
+      begin_p();
+      p32(ra[0], 0, pk);
+      p32(ra[1], 1, pk);
+    }
+    // P over the first half of S.
+    ptx::tmem_st32(tS, pk);
+    if constexpr (TILE == 128) {
+      p32(rb[0], 2, pk);
+      p32(rb[1], 3, pk);
+      ptx::tmem_st32(tS + 32, pk);
     }
     if constexpr (FSW > 0) {
       l_sum += l_tile;
@@ -708,7 +752,7 @@ __device__ __forceinline__ void softmax_epilogue(const ProbeLaunch& L, const Wor
 }
 
 template <int TILE, int D, int NS, int FSW, int EMB>
-__global__ void __launch_bounds__(kThreads, 1) probe_attn_kernel(const __grid_constant__ ProbeLaunch L) {
+__global__ void __launch_bounds__(kThreads<TILE>, 1) probe_attn_kernel(const __grid_constant__ ProbeLaunch L) {
   using C = Cfg<TILE, D, NS>;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -728,13 +772,15 @@ __global__ void __launch_bounds__(kThreads, 1) probe_attn_kernel(const __grid_co
   ptx::tc_fence_after();
   const uint32_t tmem = *tmem_slot;
 
-  if (warp == kWarpProducer) {
-    producer<TILE, D, NS, false>(L, it, sbase, abort_flag);
-  } else if (warp == kWarpVLoader) {
-    producer<TILE, D, NS, true>(L, it, sbase, abort_flag);
-  } else if (warp == kWarpMma) {
-    mma_issuer<TILE, D, NS>(L, it, sbase, tmem, abort_flag);
+  // 256 x 208 + 128 x 88 = 384 x 168 registers, what the launch holds: the
+  // softmax keeps a whole row of S and its P.
+  if (warp >= kWarpProducer) {
+    if constexpr (TILE == 128) ptx::setmaxnreg_dec<88>();
+    if (warp == kWarpProducer) producer<TILE, D, NS, false>(L, it, sbase, abort_flag);
+    else if (warp == kWarpVLoader) producer<TILE, D, NS, true>(L, it, sbase, abort_flag);
+    else if (warp == kWarpMma) mma_issuer<TILE, D, NS>(L, it, sbase, tmem, abort_flag);
   } else {
+    if constexpr (TILE == 128) ptx::setmaxnreg_inc<208>();
     softmax_epilogue<TILE, D, NS, FSW, EMB>(L, it, warp / 4, sbase, tmem, abort_flag);
   }
   ptx::tc_fence_before();
@@ -753,7 +799,7 @@ cudaError_t launch_cfg(const ProbeLaunch& L, cudaStream_t stream) {
   static PerDeviceAttr smem_once;
   cudaError_t e = raise_smem_limit(smem_once, reinterpret_cast<const void*>(kern), C::SMEM_BYTES);
   if (e != cudaSuccess) return e;
-  kern<<<L.n_items, kThreads, C::SMEM_BYTES, stream>>>(L);
+  kern<<<L.n_items, kThreads<TILE>, C::SMEM_BYTES, stream>>>(L);
   return cudaGetLastError();
 }
 
