@@ -26,8 +26,8 @@
 //               fp32 in TMEM; M = 128 keys, N = the tile's text rows). Issuing
 //               blocks while the tensor pipe is busy, so one warp's waits fall
 //               into the other's MMAs
-//   warp 19     the steps' LSEs, negated in log2 units, to shared memory; it
-//               arrives on the same barrier as the step's MMA
+//   warp 19     the steps' LSEs, negated in log2 units, to shared memory (two
+//               steps ahead); it arrives on the same barrier as the step's MMA
 // What bounds it: per (text row, key) pair one ex2 on the XU pipe (32 per clock
 // and SM) and 2 d tensor flops. A tcgen05.mma with A and B in shared memory
 // takes at least 64 clocks whatever its N (measured: 72 at N = 32, 69 at N =
@@ -36,8 +36,9 @@
 // hidden only behind other heads' sums, hence the groups.
 // A pair of columns is one packed fma, two ex2 and one packed add. The call
 // with one CTA per (128 keys, KV group), one thread per key and two CTAs per SM
-// took 415 us on the 8-video batch and 108 us on 65,664 tokens; this one 340
-// and 83 us.
+// took 415 us on the 8-video batch, 108 us on 65,664 tokens, 34 us on 16,512 and
+// 16.4 us on 4,160; this one 339, 79, 29 and 12.4 us. (The LSE warp with one
+// step's loads in flight, serialised by a branch: 397, 91, 43 and 14.5 us.)
 // Every (head, key) has one writer and a fixed summation order. Every wait is
 // bounded; on timeout the CTA records EVISEL_ETIMEOUT and drains its copies
 // and MMAs. The key warps never leave their loop early; after a timeout they
@@ -53,6 +54,7 @@ namespace {
 
 constexpr int kRows = 128;                       // keys of a unit (TMEM lanes)
 constexpr int kMaxText = 256;                    // text rows of a step
+constexpr int kUnitTable = 64;                   // units of a CTA looked up before the roles start
 constexpr int kMaxBlocks = 8;                    // mask blocks of a unit's keys (16 tokens at least)
 constexpr int kGroups = 4;                       // groups of key threads: heads in flight
 constexpr int kKeyWarps = kGroups * kRows / 32;
@@ -75,7 +77,8 @@ struct TeCfg {
   static constexpr int OFF_Q = KS * K_BYTES;
   static constexpr int OFF_LSE = OFF_Q + QS * K_BYTES;              // per S buffer [blocks of the keys][its columns] fp32
   static constexpr int OFF_RED = OFF_LSE + kMaxBlocks * kTmemCols * 4;   // [kKeyWarps] fp32
-  static constexpr int OFF_BAR = OFF_RED + kKeyWarps * 4;
+  static constexpr int OFF_UNIT = OFF_RED + kKeyWarps * 4;          // [kUnitTable] Unit
+  static constexpr int OFF_BAR = OFF_UNIT + kUnitTable * 48;
   static constexpr int B_KF = 0, B_KE = B_KF + KS, B_QF = B_KE + KS, B_QE = B_QF + QS, B_SF = B_QE + QS,
                        B_SE = B_SF + NB, B_DRAIN = B_SE + NB;
   static constexpr int N_BARS = B_DRAIN + kMmaWarps;
@@ -94,11 +97,11 @@ __device__ __forceinline__ void record_failure(volatile int* abort_flag, int* st
   atomicExch(status, kStatusTimeout);
 }
 
-// Unit u: heads [h0, h0 + nh) of KV group g against the keys [col0, col0 + 128)
+// Heads [h0, h0 + nh) of KV group g against the keys [col0, col0 + 128)
 // of a video, in nh heads x n_tt text tiles of tile_rows rows.
 struct Unit {
   int col0, vis_start, n_vis, n_text, vis_off, frame_off;
-  int g, h0, nh, n_tt, tile_rows;
+  int g, h0, nh, n_tt, tile_rows, pad;
 };
 
 __device__ __forceinline__ Unit unit_of(const TextEvidenceLaunch& L, int u) {
@@ -118,11 +121,13 @@ __device__ __forceinline__ Unit unit_of(const TextEvidenceLaunch& L, int u) {
   x.vis_off = vi.vis_off;
   x.frame_off = vi.frame_off;
   x.n_tt = (x.n_text + L.text_cols - 1) / L.text_cols;
+  x.pad = 0;
   x.tile_rows = x.n_tt > 0 ? ((x.n_text + x.n_tt - 1) / x.n_tt + 15) & ~15 : 0;   // at most text_cols
   return x;
 }
 
-template <int D>
+// kKeep: the probe ran with per-row block masks.
+template <int D, bool kKeep>
 __global__ void __launch_bounds__(kThreads, 1) text_evidence_kernel(const __grid_constant__ TextEvidenceLaunch L) {
   using C = TeCfg<D>;
   extern __shared__ uint8_t smem_raw[];
@@ -135,7 +140,7 @@ __global__ void __launch_bounds__(kThreads, 1) text_evidence_kernel(const __grid
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int n_units = L.n_chunks * L.hkv * L.head_split;
   const int nb = kTmemCols / L.text_cols;          // S buffers = groups in use
-  const int nblk = L.keep ? kRows / L.keep_block : 1;   // mask blocks of a unit's keys
+  const int nblk = kKeep ? kRows / L.keep_block : 1;   // mask blocks of a unit's keys
   // The n-th Q tile of MMA warp w is in stage w spw + n % spw, phase n / spw:
   // every barrier has one waiter, which sees each of its phases (a parity wait
   // must never run two phases ahead).
@@ -151,6 +156,18 @@ __global__ void __launch_bounds__(kThreads, 1) text_evidence_kernel(const __grid
     return free_;
   };
 
+  // The CTA's units, looked up in parallel: two dependent global loads per unit
+  // and role would cost more than a short unit's sums.
+  Unit* table = reinterpret_cast<Unit*>(smem + C::OFF_UNIT);
+  static_assert(sizeof(Unit) == 48 && C::OFF_UNIT % 16 == 0, "unit table");
+  if (threadIdx.x >= 64 && threadIdx.x < 64 + kUnitTable) {
+    const int i = threadIdx.x - 64, u = blockIdx.x + i * gridDim.x;
+    if (u < n_units) table[i] = unit_of(L, u);
+  }
+  auto unit_at = [&](int u) -> Unit {
+    const int i = (u - static_cast<int>(blockIdx.x)) / static_cast<int>(gridDim.x);
+    return i < kUnitTable ? table[i] : unit_of(L, u);
+  };
   if (threadIdx.x == 0) {
     for (int i = 0; i < C::N_BARS; ++i)
       ptx::mbar_init(bar(i), i >= C::B_SF && i < C::B_SF + C::NB   ? 2u     // the MMA's commit and the LSE warp
@@ -177,7 +194,7 @@ __global__ void __launch_bounds__(kThreads, 1) text_evidence_kernel(const __grid
     int nk = 0, nh = 0;                          // K tiles issued, heads so far
     int nq[kMmaWarps] = {};                      // Q tiles issued to each MMA warp
     for (int u = blockIdx.x; ok && u < n_units; u += gridDim.x) {
-      const Unit x = unit_of(L, u);
+      const Unit x = unit_at(u);
       if (x.n_tt == 0) continue;                 // a video without text rows: nothing to load
       const int ks = nk % C::KS;
       if (nk >= C::KS && !warp_wait(bar(C::B_KE + ks), ((nk - C::KS) / C::KS) & 1, abort_flag)) {
@@ -235,7 +252,7 @@ __global__ void __launch_bounds__(kThreads, 1) text_evidence_kernel(const __grid
     const uint64_t dk = ptx::sdesc_sw128(sbase + C::OFF_K, 16, 1024);
     const uint64_t dq = ptx::sdesc_sw128(sbase + C::OFF_Q, 16, 1024);
     for (int u = blockIdx.x; ok && u < n_units; u += gridDim.x) {
-      const Unit x = unit_of(L, u);
+      const Unit x = unit_at(u);
       if (x.n_tt == 0) continue;
       const int ks = nk % C::KS;
       if (!warp_wait(bar(C::B_KF + ks), (nk / C::KS) & 1, abort_flag)) {
@@ -295,44 +312,41 @@ __global__ void __launch_bounds__(kThreads, 1) text_evidence_kernel(const __grid
     __syncwarp();
   } else if (warp == kWarpLse) {
     // Per step: -LSE log2e of the tile's text rows, -inf past the tile's rows
-    // or the video's text (those columns add 0). The next step's values are
-    // loaded before this step's wait.
+    // or the video's text (those columns add 0). Two steps' values are in
+    // flight while a third one waits for its buffer: a step takes less time
+    // than a load.
+    struct Step {
+      float lse[kMaxText / 32];
+      uint32_t bits[kKeep ? kMaxText / 32 : 1];    // per row: bit i = the unit's i-th block is kept
+      int rows, buf;
+      bool valid;
+    };
     int u = blockIdx.x, hh = 0, tt = 0, nh = 0;
     Unit x{};
     auto seek = [&]() {                            // the next unit with text rows
       for (; u < n_units; u += gridDim.x) {
-        x = unit_of(L, u);
+        x = unit_at(u);
         if (x.n_tt > 0) return;
       }
     };
-    float next[kMaxText / 32];
-    uint32_t bits[kMaxText / 32];                  // per row: bit i = the unit's i-th block is kept
-    auto load = [&]() {
+    auto load = [&](Step& s) {
+      s.valid = u < n_units;
+      if (!s.valid) return;
+      s.rows = x.tile_rows;
+      s.buf = nh & (nb - 1);
       const float* lse = L.lse + static_cast<int64_t>(x.h0 + hh) * L.n_tok + x.vis_start + x.n_vis;
 #pragma unroll
       for (int i = 0; i < kMaxText / 32; ++i) {
         const int r = i * 32 + lane, row = tt * x.tile_rows + r;
         const bool in = r < x.tile_rows && row < x.n_text;
-        next[i] = in ? -1.4426950408889634f * __ldg(lse + row) : -INFINITY;
-        bits[i] = 1u;
-        if (L.keep && in) {
+        s.lse[i] = in ? __ldg(lse + row) : INFINITY;   // (no branch and no use here: the loads overlap)
+        if constexpr (kKeep) {
           const int blk0 = x.col0 / L.keep_block;  // a multiple of nblk: the blocks share one word
-          bits[i] = __ldg(L.keep + (static_cast<int64_t>(x.h0 + hh) * L.keep_words + (blk0 >> 5)) * L.n_tok +
-                          x.vis_start + x.n_vis + row) >> (blk0 & 31);
+          s.bits[i] = in ? __ldg(L.keep + (static_cast<int64_t>(x.h0 + hh) * L.keep_words + (blk0 >> 5)) * L.n_tok +
+                                 x.vis_start + x.n_vis + row) >> (blk0 & 31)
+                         : 0u;
         }
       }
-    };
-    seek();
-    if (u < n_units) load();
-    while (u < n_units) {
-      float cur[kMaxText / 32];
-      uint32_t cur_bits[kMaxText / 32];
-#pragma unroll
-      for (int i = 0; i < kMaxText / 32; ++i) {
-        cur[i] = next[i];
-        cur_bits[i] = bits[i];
-      }
-      const int b = nh & (nb - 1);
       if (++tt == x.n_tt) {
         tt = 0;
         ++nh;
@@ -342,19 +356,38 @@ __global__ void __launch_bounds__(kThreads, 1) text_evidence_kernel(const __grid
           seek();
         }
       }
-      if (u < n_units) load();
-      if (!buffer_free(b)) {
+    };
+    auto put = [&](const Step& s) {
+      if (!buffer_free(s.buf)) {
         ok = false;
-        break;
+        return;
       }
       for (int kb = 0; kb < nblk; ++kb) {
-        float* row = lse_s + (b * nblk + kb) * L.text_cols;
+        float* row = lse_s + (s.buf * nblk + kb) * L.text_cols;
 #pragma unroll
         for (int i = 0; i < kMaxText / 32; ++i)
-          if (i * 32 < L.text_cols) row[i * 32 + lane] = (cur_bits[i] >> kb) & 1u ? cur[i] : -INFINITY;
+          if (i * 32 < s.rows) {
+            const float v = -1.4426950408889634f * s.lse[i];
+            if constexpr (kKeep) row[i * 32 + lane] = (s.bits[i] >> kb) & 1u ? v : -INFINITY;
+            else row[i * 32 + lane] = v;
+          }
       }
       __syncwarp();
-      if (lane == 0) ptx::mbar_arrive(bar(C::B_SF + b));
+      if (lane == 0) ptx::mbar_arrive(bar(C::B_SF + s.buf));
+    };
+    seek();
+    Step s0, s1, s2;
+    load(s0);
+    load(s1);
+    while (ok && s0.valid) {
+      load(s2);
+      put(s0);
+      if (!ok || !s1.valid) break;
+      load(s0);
+      put(s1);
+      if (!ok || !s2.valid) break;
+      load(s1);
+      put(s2);
     }
     if (!ok && lane == 0) record_failure(abort_flag, L.status);
   } else {
@@ -365,12 +398,12 @@ __global__ void __launch_bounds__(kThreads, 1) text_evidence_kernel(const __grid
     const uint64_t scale2 = ptx::f2(L.scale_log2, L.scale_log2);
     const int npf = L.tokens_per_frame, w = npf < 32 ? npf : 32;
     const int log_npf = 31 - __clz(npf);           // N_v is a power of two
-    const int kblk = L.keep ? key / L.keep_block : 0;   // the key's mask block within the unit
+    const int kblk = kKeep ? key / L.keep_block : 0;   // the key's mask block within the unit
     float* red = reinterpret_cast<float*>(smem + C::OFF_RED);
     int nh = 0;                                    // heads of this CTA so far
     uint32_t step = 0;                             // steps of this group so far
     for (int u = blockIdx.x; u < n_units && grp < nb; u += gridDim.x) {
-      const Unit x = unit_of(L, u);
+      const Unit x = unit_at(u);
       const int nkeys = min(kRows, x.n_vis - x.col0);   // a multiple of N_v
       const bool warp_ok = (warp & 3) * 32 < nkeys;     // some key of the warp exists
       for (int hh = 0; hh < x.nh; ++hh) {
@@ -452,10 +485,10 @@ __global__ void __launch_bounds__(kThreads, 1) text_evidence_kernel(const __grid
   }
 }
 
-template <int D>
+template <int D, bool kKeep>
 cudaError_t launch_d(const TextEvidenceLaunch& L, cudaStream_t stream) {
   using C = TeCfg<D>;
-  auto kern = text_evidence_kernel<D>;
+  auto kern = text_evidence_kernel<D, kKeep>;
   static PerDeviceAttr smem_once;
   cudaError_t e = raise_smem_limit(smem_once, reinterpret_cast<const void*>(kern), C::SMEM_BYTES);
   if (e != cudaSuccess) return e;
@@ -487,8 +520,8 @@ cudaError_t launch_d(const TextEvidenceLaunch& L, cudaStream_t stream) {
 
 cudaError_t launch_text_evidence(const TextEvidenceLaunch& L, cudaStream_t stream) {
   if (L.n_chunks == 0) return cudaSuccess;
-  if (L.head_dim == 128) return launch_d<128>(L, stream);
-  if (L.head_dim == 64) return launch_d<64>(L, stream);
+  if (L.head_dim == 128) return L.keep ? launch_d<128, true>(L, stream) : launch_d<128, false>(L, stream);
+  if (L.head_dim == 64) return L.keep ? launch_d<64, true>(L, stream) : launch_d<64, false>(L, stream);
   return cudaErrorInvalidValue;
 }
 
