@@ -306,8 +306,7 @@ int evisel_topp_mask(const evisel_probe_args* args, int32_t block, float tau_p, 
  *          by about hq * n_text_total * 32 * W * 4 bytes).
  *   accumulate  0: overwrite tok and frame; 1: add (sum over layers); head and
  *          aqf are recomputed from the resulting frame map.
- * Asynchronous on `stream` after a short synchronous upload of the per-video
- * offsets. Errors: EVISEL_EINVAL, EVISEL_ESTATE (no evisel_topp_mask on ws),
+ * Asynchronous on `stream`. Errors: EVISEL_EINVAL, EVISEL_ESTATE (no evisel_topp_mask on ws),
  * EVISEL_ENOMEM, EVISEL_ECUDA. */
 int evisel_coarse_evidence(const evisel_probe_args* args, evisel_ws* ws, int32_t block, const uint32_t* keep,
                            float* tok, float* frame, float* head, float* aqf, int accumulate, void* stream);

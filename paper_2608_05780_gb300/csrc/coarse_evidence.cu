@@ -7,27 +7,34 @@
 // visual tokens m, frame sums, head sums and A_qf. All tokens of a retained
 // visual block share its weight exp(g_ij - M_i) / Z_i.
 //
-// coarse_rows_kernel: one CTA per (8 text rows of a video, head), a warp per
-//   row. The CTA stages the k_bar rows of the head's KV group in chunks of 32
-//   blocks (one keep word) in shared memory; lane j of a warp takes block
-//   j of each chunk: it forms g_ij = scale q_i k_bar_j (stored for the next
-//   kernel) and, over its blocks in S_i, a running max and sum. The lanes'
-//   pairs then merge (a butterfly: each step's merge is symmetric, so all
-//   lanes agree) and the warp adds the exact logits s of the own block's
-//   causal prefix E_i, giving M_i and
-//   Z_i = sum_{S_i} B exp(g - M) + sum_{E_i} exp(s - M).
-// coarse_map_kernel: one thread per (frame, head, video): for each block of
-//   the frame, c_j = sum over the video's text rows of [j in S_i]
-//   exp(g_ij - M_i) / Z_i (rows in order: deterministic); writes c_j to the
-//   block's tokens and B sum_j c_j to the frame.
-// coarse_finalize_kernel: head[b, h] = sum of the video's frames; A_qf[t] =
-//   sum_h frame[h, t] / (Hq n_text), from the (possibly accumulated) frame map.
-#include <algorithm>
+// coarse_logits_kernel: one CTA per (16 text rows of a video, 256 blocks, head):
+//   a lane takes one block for all 16 rows, so that its k_bar values are
+//   converted once; the rows' q sit in shared memory as fp32 (broadcast reads),
+//   two dims per packed fma. Writes g_ij = scale q_i k_bar_j.
+// coarse_rows_kernel: a warp per (text row, head): a running max and sum over
+//   the row's retained blocks (B tokens each) and over the exact logits s of
+//   its own block's causal prefix E_i (a lane per key), merged over the lanes:
+//   M_i and Z_i = sum_{S_i} B exp(g - M) + sum_{E_i} exp(s - M).
+// coarse_map_kernel: one CTA per (32 visual blocks, head): a lane per block, the
+//   text rows dealt over eight warps whose sums meet in shared memory in warp
+//   order (deterministic): c_j = sum over the video's text rows of [j in S_i]
+//   exp(g_ij - M_i) / Z_i; writes c_j to the block's tokens and B sum_j c_j to
+//   the frame.
+// coarse_finalize_kernel: head[b, h] = sum of the video's frames (a warp each);
+//   A_qf[t] = sum_h frame[h, t] / (Hq n_text) (a thread per frame), from the
+//   (possibly accumulated) frame map.
+// What bounds it: a few MB and under 1 GFLOP, so latency: serial loops over a
+// row's own keys (a load and a warp sum per key), over the text rows of a frame
+// in one thread and over a head's frames in one thread took 64, 40 and 15 us on
+// 16,388 tokens (28 heads, 100 text rows, B = 32); here the logits, rows, map and
+//   finalize kernels take 22, 14, 9 and 3 us, the call 137 -> 56 us (its per-video
+//   offsets now come with the builder's upload: no copy, no synchronisation).
 #include <cstdint>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
 #include "evisel_internal.h"
+#include "sm103_ptx.cuh"
 
 namespace evisel {
 namespace {
@@ -39,17 +46,9 @@ __device__ __forceinline__ float warp_sum(float x) {
   return x;
 }
 
-// s + sum of the 8 bf16 products of a and b, in order.
-__device__ __forceinline__ float dot8(const uint4& a, const uint4& b, float s) {
-  const __nv_bfloat162* a2 = reinterpret_cast<const __nv_bfloat162*>(&a);
-  const __nv_bfloat162* b2 = reinterpret_cast<const __nv_bfloat162*>(&b);
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const float2 fa = __bfloat1622float2(a2[i]), fb = __bfloat1622float2(b2[i]);
-    s = fmaf(fa.x, fb.x, s);
-    s = fmaf(fa.y, fb.y, s);
-  }
-  return s;
+// Two bf16 values as a packed pair of fp32.
+__device__ __forceinline__ uint64_t up2(uint32_t x) {
+  return ptx::f2(__uint_as_float(x << 16), __uint_as_float(x & 0xffff0000u));
 }
 
 // (m, z) <- the softmax pair of (m, z) and (m2, z2): max and rescaled sum.
@@ -59,92 +58,147 @@ __device__ __forceinline__ void merge_mz(float& m, float& z, float m2, float z2)
   m = mm;
 }
 
-constexpr int kRowsPerCta = 8;                   // text rows (warps) per CTA
-constexpr int kChunk = 32;                       // k_bar rows staged at a time: one keep word
+// The text rows in groups of `per` per video, videos back to back: the video
+// and group of global index i (false past the last group).
+__device__ __forceinline__ bool row_group(const CoarseLaunch& L, int i, int per, int& v, int& grp) {
+  for (v = 0; v < L.n_videos; ++v) {
+    const int n = (L.vids[v].n_text + per - 1) / per;
+    if (i < n) {
+      grp = i;
+      return true;
+    }
+    i -= n;
+  }
+  return false;
+}
 
-__global__ void __launch_bounds__(256) coarse_rows_kernel(const __grid_constant__ CoarseLaunch L) {
-  __shared__ __align__(16) __nv_bfloat16 q_s[kRowsPerCta][128];   // each warp's query row
-  __shared__ uint4 kb_s[kChunk][128 / 8 + 1];                     // k_bar rows, padded by 16 B
+constexpr int kLogitRows = 16;                   // text rows per CTA of the logits
+constexpr int kLogitBlocks = 256;                // blocks per CTA (32 per warp)
+
+template <int D>
+__global__ void __launch_bounds__(256) coarse_logits_kernel(const __grid_constant__ CoarseLaunch L) {
+  __shared__ __align__(16) float q_s[kLogitRows][D];
+  const int h = blockIdx.z;
+  int v, grp;
+  if (!row_group(L, blockIdx.y, kLogitRows, v, grp)) return;   // CTA-uniform
+  const ToppVideo vid = L.vids[v];
+  const int row0 = grp * kLogitRows, nr = min(kLogitRows, vid.n_text - row0);
+  const int B = L.block, nvb = vid.n_vis / B;
+  const int nh = nvb + (row0 + nr - 1) / B;      // blocks that end before the group's last row
+  if (static_cast<int>(blockIdx.x) * kLogitBlocks >= nh) return;
+  const __nv_bfloat16* q = static_cast<const __nv_bfloat16*>(L.q);
+  for (int i = threadIdx.x; i < kLogitRows * D; i += blockDim.x) {
+    const int r = i / D, e = i % D;
+    q_s[r][e] = r < nr ? __bfloat162float(q[(static_cast<int64_t>(vid.start + vid.n_vis + row0 + r) * L.hq + h) * D + e]) : 0.f;
+  }
+  __syncthreads();
+  const int j = blockIdx.x * kLogitBlocks + threadIdx.x;
+  if (j >= nh) return;
+  const int g = h / (L.hq / L.hkv);
+  const uint4* kb = reinterpret_cast<const uint4*>(static_cast<const __nv_bfloat16*>(L.kbar) +
+                                                   (static_cast<int64_t>(vid.blk_off + j) * L.hkv + g) * D);
+  uint64_t acc[kLogitRows];
+#pragma unroll
+  for (int r = 0; r < kLogitRows; ++r) acc[r] = 0;
+#pragma unroll 4
+  for (int c = 0; c < D / 8; ++c) {
+    const uint4 x = __ldg(kb + c);
+    const uint64_t k0 = up2(x.x), k1 = up2(x.y), k2 = up2(x.z), k3 = up2(x.w);
+#pragma unroll
+    for (int r = 0; r < kLogitRows; ++r) {
+      const ulonglong2 a = *reinterpret_cast<const ulonglong2*>(&q_s[r][c * 8]);
+      const ulonglong2 b = *reinterpret_cast<const ulonglong2*>(&q_s[r][c * 8 + 4]);
+      acc[r] = ptx::fma2(a.x, k0, acc[r]);
+      acc[r] = ptx::fma2(a.y, k1, acc[r]);
+      acc[r] = ptx::fma2(b.x, k2, acc[r]);
+      acc[r] = ptx::fma2(b.y, k3, acc[r]);
+    }
+  }
+  float* out = L.gbuf + (static_cast<int64_t>(h) * L.total_text + vid.text_off + row0) * L.pitch + j;
+#pragma unroll
+  for (int r = 0; r < kLogitRows; ++r) {
+    float lo, hi;
+    ptx::unf2(acc[r], lo, hi);
+    if (r < nr) out[static_cast<int64_t>(r) * L.pitch] = (lo + hi) * L.scale;
+  }
+}
+
+constexpr int kRowsPerCta = 8;                   // text rows (warps) per CTA
+
+template <int D>
+__global__ void __launch_bounds__(kRowsPerCta * 32) coarse_rows_kernel(const __grid_constant__ CoarseLaunch L) {
+  __shared__ __align__(16) float q_s[kRowsPerCta][D];
   const int wib = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int h = blockIdx.y;
-  // This CTA's video and row group (groups of 8 text rows, videos back to back).
-  int v = 0, grp = blockIdx.x;
-  for (; v < L.n_videos; ++v) {
-    const int cnt = (L.text_off[v + 1] - L.text_off[v] + kRowsPerCta - 1) / kRowsPerCta;
-    if (grp < cnt) break;
-    grp -= cnt;
-  }
-  if (v >= L.n_videos) return;                   // CTA-uniform, before any barrier
+  int v, grp;
+  if (!row_group(L, blockIdx.x, kRowsPerCta, v, grp)) return;
   const ToppVideo vid = L.vids[v];
-  const int n_text = L.text_off[v + 1] - L.text_off[v];
-  const int t_last = min(grp * kRowsPerCta + kRowsPerCta - 1, n_text - 1);
-  const int t = min(grp * kRowsPerCta + wib, t_last);   // text row within the video (clamped)
-  const bool active = grp * kRowsPerCta + wib <= t_last;   // warp-uniform
-  const int trow = L.text_off[v] + t;            // text row over all videos
+  const int t = grp * kRowsPerCta + wib;         // text row within the video
+  if (t >= vid.n_text) return;                   // warp-uniform; no CTA barrier below
+  const int trow = vid.text_off + t;             // text row over all videos
   const int pos = vid.n_vis + t;                 // video-local position
   const int row = vid.start + pos;               // global token
-  const int B = L.block, nvb = vid.n_vis / B;
-  const int nh = nvb + t / B;                    // blocks that end before the row
-  const int nh_cta = nvb + t_last / B;           // the most over the CTA's rows
+  const int B = L.block;
+  const int nh = vid.n_vis / B + t / B;          // blocks that end before the row
   const int own0 = vid.n_vis + (t / B) * B;      // first token of its own block
   const int g = h / (L.hq / L.hkv);
-  const int d = L.head_dim, dc = d / 8;          // d = 64 or 128
-  const __nv_bfloat16* q = static_cast<const __nv_bfloat16*>(L.q) + (static_cast<int64_t>(row) * L.hq + h) * d;
-  for (int c = lane; c < dc; c += 32) reinterpret_cast<uint4*>(q_s[wib])[c] = reinterpret_cast<const uint4*>(q)[c];
+  const __nv_bfloat16* q = static_cast<const __nv_bfloat16*>(L.q) + (static_cast<int64_t>(row) * L.hq + h) * D;
+  for (int e = lane; e < D; e += 32) q_s[wib][e] = __bfloat162float(q[e]);
   __syncwarp();
-  const uint4* q4 = reinterpret_cast<const uint4*>(q_s[wib]);
-  const __nv_bfloat16* kbar = static_cast<const __nv_bfloat16*>(L.kbar);
-  const __nv_bfloat16* k = static_cast<const __nv_bfloat16*>(L.k);
-  float* grow = L.gbuf + (static_cast<int64_t>(h) * L.total_text + trow) * L.pitch;
-  const uint32_t* keep = L.keep + static_cast<int64_t>(h) * L.n_words * L.n_tok + row;
   float m = -INFINITY, z = 0.f;
-  for (int j0 = 0; j0 < nh_cta; j0 += kChunk) {
-    __syncthreads();                             // the previous chunk is consumed
-    for (int i = threadIdx.x; i < kChunk * dc; i += blockDim.x) {   // coalesced: 16 B per thread
-      const int jj = i / dc, c = i % dc;
-      if (j0 + jj < nh_cta)
-        kb_s[jj][c] = reinterpret_cast<const uint4*>(kbar + (static_cast<int64_t>(vid.blk_off + j0 + jj) * L.hkv + g) * d)[c];
+  auto add = [&](float x, float n) {             // n tokens of logit x
+    if (x > m) {
+      z = (m == -INFINITY) ? 0.f : z * __expf(m - x);
+      m = x;
     }
-    __syncthreads();
-    const int j = j0 + lane;
-    if (active && j < nh) {
-      const uint32_t word = keep[static_cast<int64_t>(j0 >> 5) * L.n_tok];
-      float s = 0.f;
-      for (int c = 0; c < dc; ++c) s = dot8(q4[c], kb_s[lane][c], s);
-      const float gj = s * L.scale;
-      grow[j] = gj;
-      if ((word >> lane) & 1u) {                 // j in S_i: B tokens share g_ij
-        if (gj > m) {
-          z = (m == -INFINITY) ? 0.f : z * __expf(m - gj);
-          m = gj;
-        }
-        z += static_cast<float>(B) * __expf(gj - m);
-      }
+    z += n * __expf(x - m);
+  };
+  // S_i: the row's retained blocks, eight words at a time.
+  const float* grow = L.gbuf + (static_cast<int64_t>(h) * L.total_text + trow) * L.pitch;
+  const uint32_t* keep = L.keep + static_cast<int64_t>(h) * L.n_words * L.n_tok + row;
+  for (int w0 = 0; w0 * 32 < nh; w0 += 8) {
+    float x[8];
+    uint32_t word[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int j = (w0 + i) * 32 + lane;
+      x[i] = j < nh ? grow[j] : 0.f;
+      word[i] = (w0 + i) * 32 < nh ? __ldg(keep + static_cast<int64_t>(w0 + i) * L.n_tok) : 0u;
     }
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+      if ((w0 + i) * 32 + lane < nh && ((word[i] >> lane) & 1u)) add(x[i], static_cast<float>(B));
   }
-  if (!active) return;                           // warp-uniform; no barrier follows
-  for (int off = 16; off > 0; off >>= 1) {
+  // E_i: exact logits of the own block's causal prefix, a lane per key.
+  const __nv_bfloat16* k = static_cast<const __nv_bfloat16*>(L.k);
+  const bool aligned = (reinterpret_cast<uintptr_t>(k) & 15u) == 0;   // (the caller's k; k_bar is the workspace's)
+  for (int mm = own0 + lane; mm <= pos; mm += 32) {
+    const __nv_bfloat16* kr = k + (static_cast<int64_t>(vid.start + mm) * L.hkv + g) * D;
+    auto load8 = [&](int c) {
+      if (aligned) return __ldg(reinterpret_cast<const uint4*>(kr) + c);
+      const uint16_t* e = reinterpret_cast<const uint16_t*>(kr) + c * 8;
+      return make_uint4(e[0] | e[1] << 16, e[2] | e[3] << 16, e[4] | e[5] << 16, e[6] | e[7] << 16);
+    };
+    uint64_t acc[2] = {0, 0};
+#pragma unroll 4
+    for (int c = 0; c < D / 8; ++c) {
+      const uint4 x = load8(c);
+      const ulonglong2 a = *reinterpret_cast<const ulonglong2*>(&q_s[wib][c * 8]);
+      const ulonglong2 b = *reinterpret_cast<const ulonglong2*>(&q_s[wib][c * 8 + 4]);
+      acc[0] = ptx::fma2(a.x, up2(x.x), acc[0]);
+      acc[1] = ptx::fma2(a.y, up2(x.y), acc[1]);
+      acc[0] = ptx::fma2(b.x, up2(x.z), acc[0]);
+      acc[1] = ptx::fma2(b.y, up2(x.w), acc[1]);
+    }
+    float s0, s1, s2, s3;
+    ptx::unf2(acc[0], s0, s1);
+    ptx::unf2(acc[1], s2, s3);
+    add(((s0 + s1) + (s2 + s3)) * L.scale, 1.f);
+  }
+  __syncwarp();
+  for (int off = 16; off > 0; off >>= 1) {       // symmetric merges: all lanes agree
     const float m2 = __shfl_xor_sync(kFull, m, off), z2 = __shfl_xor_sync(kFull, z, off);
     merge_mz(m, z, m2, z2);
-  }
-  // E_i: exact logits of the own block's causal prefix; lanes split d.
-  const int per = d / 32;
-  float qv[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-  for (int e = 0; e < 4; ++e)
-    if (e < per) qv[e] = __bfloat162float(q_s[wib][lane * per + e]);
-  for (int mm = own0; mm <= pos; ++mm) {
-    const __nv_bfloat16* kr = k + (static_cast<int64_t>(vid.start + mm) * L.hkv + g) * d;
-    float s = 0.f;
-#pragma unroll
-    for (int e = 0; e < 4; ++e)
-      if (e < per) s += qv[e] * __bfloat162float(kr[lane * per + e]);
-    s = warp_sum(s) * L.scale;
-    if (s > m) {
-      z = (m == -INFINITY) ? 0.f : z * __expf(m - s);
-      m = s;
-    }
-    z += __expf(s - m);
   }
   if (lane == 0) {
     L.row_m[static_cast<int64_t>(h) * L.total_text + trow] = m;
@@ -152,75 +206,123 @@ __global__ void __launch_bounds__(256) coarse_rows_kernel(const __grid_constant_
   }
 }
 
-__global__ void __launch_bounds__(128) coarse_map_kernel(const __grid_constant__ CoarseLaunch L) {
-  const int v = blockIdx.z, h = blockIdx.y;
-  const ToppVideo vid = L.vids[v];
+constexpr int kMapWarps = 8;
+
+__global__ void __launch_bounds__(kMapWarps * 32) coarse_map_kernel(const __grid_constant__ CoarseLaunch L) {
+  __shared__ float part[kMapWarps][32];
+  __shared__ float c_s[32];
+  const int h = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int npf = L.tokens_per_frame, B = L.block;
-  const int n_frames = vid.n_vis / npf;
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= n_frames) return;
-  const int n_text = vid.n_text;
-  const int tr0 = L.text_off[v];
-  float fsum = 0.f;
-  for (int jj = 0; jj < npf / B; ++jj) {
-    const int j = t * (npf / B) + jj;            // visual block
-    float c = 0.f;
-    for (int i = 0; i < n_text; ++i) {
-      const int row = vid.start + vid.n_vis + i;
-      const uint32_t word = L.keep[(static_cast<int64_t>(h) * L.n_words + (j >> 5)) * L.n_tok + row];
-      if ((word >> (j & 31)) & 1u) {
-        const int64_t r = static_cast<int64_t>(h) * L.total_text + tr0 + i;
-        c += __expf(L.gbuf[r * L.pitch + j] - L.row_m[r]) / L.row_z[r];
-      }
-    }
-    float* tok = L.tok + static_cast<int64_t>(h) * L.total_vis + L.vis_off[v] + j * B;
-    for (int e = 0; e < B; ++e) tok[e] = L.accumulate ? tok[e] + c : c;
-    fsum += static_cast<float>(B) * c;
+  int v = 0, chunk = blockIdx.x;                 // chunks of 32 visual blocks, videos back to back
+  for (; v < L.n_videos; ++v) {
+    const int n = (L.vids[v].n_vis / B + 31) / 32;
+    if (chunk < n) break;
+    chunk -= n;
   }
-  float* fr = L.frame + static_cast<int64_t>(h) * L.total_frames + L.frame_off[v] + t;
-  *fr = L.accumulate ? *fr + fsum : fsum;
+  if (v >= L.n_videos) return;                   // CTA-uniform
+  const ToppVideo vid = L.vids[v];
+  const int j0 = chunk * 32, nb = min(32, vid.n_vis / B - j0);
+  const int64_t r0 = static_cast<int64_t>(h) * L.total_text + vid.text_off;
+  const float* gcol = L.gbuf + r0 * L.pitch + j0 + lane;
+  const uint32_t* keep = L.keep + (static_cast<int64_t>(h) * L.n_words + chunk) * L.n_tok + vid.start + vid.n_vis;
+  float c = 0.f;
+#pragma unroll 4
+  for (int i = warp; i < vid.n_text; i += kMapWarps) {
+    const uint32_t word = __ldg(keep + i);
+    const float x = lane < nb ? gcol[static_cast<int64_t>(i) * L.pitch] : 0.f;
+    const float m = L.row_m[r0 + i], z = L.row_z[r0 + i];
+    if (lane < nb && ((word >> lane) & 1u)) c += __expf(x - m) / z;
+  }
+  part[warp][lane] = c;
+  __syncthreads();
+  if (warp == 0) {
+    float s = 0.f;
+#pragma unroll
+    for (int w = 0; w < kMapWarps; ++w) s += part[w][lane];
+    c_s[lane] = s;
+  }
+  __syncthreads();
+  float* tok = L.tok + static_cast<int64_t>(h) * L.total_vis + vid.vis_off + static_cast<int64_t>(j0) * B;
+  for (int i = threadIdx.x; i < nb * B; i += blockDim.x) tok[i] = L.accumulate ? tok[i] + c_s[i / B] : c_s[i / B];
+  const int per = npf / B;                       // blocks per frame: 1 .. 8, so frames stay in a chunk
+  if (threadIdx.x < nb / per) {
+    float f = 0.f;
+    for (int i = 0; i < per; ++i) f += static_cast<float>(B) * c_s[threadIdx.x * per + i];
+    float* fr = L.frame + static_cast<int64_t>(h) * L.total_frames + vid.vis_off / npf + j0 / per + threadIdx.x;
+    *fr = L.accumulate ? *fr + f : f;
+  }
 }
 
-__global__ void __launch_bounds__(128) coarse_finalize_kernel(const __grid_constant__ CoarseLaunch L) {
-  const int v = blockIdx.y;
-  const ToppVideo vid = L.vids[v];
-  const int n_frames = vid.n_vis / L.tokens_per_frame;
-  const int f0 = L.frame_off[v];
-  if (blockIdx.x == 0) {                         // head map: one thread per head
-    for (int h = threadIdx.x; h < L.hq; h += blockDim.x) {
-      float s = 0.f;
-      for (int t = 0; t < n_frames; ++t) s += L.frame[static_cast<int64_t>(h) * L.total_frames + f0 + t];
-      L.head[static_cast<int64_t>(v) * L.hq + h] = s;
+constexpr int kFinalWarps = 8;
+
+// Blocks [0, n_videos * head_blocks): a warp per (video, head); then a thread per frame.
+__global__ void __launch_bounds__(kFinalWarps * 32) coarse_finalize_kernel(const __grid_constant__ CoarseLaunch L,
+                                                                          int head_blocks) {
+  const int npf = L.tokens_per_frame;
+  if (static_cast<int>(blockIdx.x) < L.n_videos * head_blocks) {
+    const int v = blockIdx.x / head_blocks, lane = threadIdx.x & 31;
+    const int h = (blockIdx.x % head_blocks) * kFinalWarps + (threadIdx.x >> 5);
+    if (h >= L.hq) return;
+    const ToppVideo vid = L.vids[v];
+    const int frames = vid.n_vis / npf;
+    const float* fr = L.frame + static_cast<int64_t>(h) * L.total_frames + vid.vis_off / npf;
+    float s[4] = {0.f, 0.f, 0.f, 0.f};
+    int t = lane;
+    for (; t + 96 < frames; t += 128) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) s[i] += fr[t + 32 * i];
     }
+    for (; t < frames; t += 32) s[0] += fr[t];
+    const float sum = warp_sum((s[0] + s[1]) + (s[2] + s[3]));
+    if (lane == 0) L.head[static_cast<int64_t>(v) * L.hq + h] = sum;
+    return;
   }
-  const float inv = vid.n_text > 0 ? 1.f / (static_cast<float>(L.hq) * vid.n_text) : 0.f;
-  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n_frames; t += gridDim.x * blockDim.x) {
-    float s = 0.f;
-    for (int h = 0; h < L.hq; ++h) s += L.frame[static_cast<int64_t>(h) * L.total_frames + f0 + t];
-    L.aqf[f0 + t] = s * inv;
+  const int t = (blockIdx.x - L.n_videos * head_blocks) * blockDim.x + threadIdx.x;
+  if (t >= L.total_frames) return;
+  int v = 0;                                     // the video that owns frame t
+  while (v + 1 < L.n_videos && L.vids[v + 1].vis_off / npf <= t) ++v;
+  const int n_text = L.vids[v].n_text;
+  float s0 = 0.f, s1 = 0.f;
+#pragma unroll 4
+  for (int h = 0; h + 1 < L.hq; h += 2) {
+    s0 += L.frame[static_cast<int64_t>(h) * L.total_frames + t];
+    s1 += L.frame[static_cast<int64_t>(h + 1) * L.total_frames + t];
   }
+  if (L.hq & 1) s0 += L.frame[static_cast<int64_t>(L.hq - 1) * L.total_frames + t];
+  L.aqf[t] = n_text > 0 ? (s0 + s1) / (static_cast<float>(L.hq) * static_cast<float>(n_text)) : 0.f;
+}
+
+template <int D>
+cudaError_t launch_rows(const CoarseLaunch& L, cudaStream_t stream) {
+  // Row groups per video: at most total / size full ones and a partial one per
+  // video; CTAs past the last group return at once.
+  dim3 g1((L.max_blocks + kLogitBlocks - 1) / kLogitBlocks, L.total_text / kLogitRows + L.n_videos, L.hq);
+  coarse_logits_kernel<D><<<g1, 256, 0, stream>>>(L);
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  dim3 g2(L.total_text / kRowsPerCta + L.n_videos, L.hq);
+  coarse_rows_kernel<D><<<g2, kRowsPerCta * 32, 0, stream>>>(L);
+  return cudaGetLastError();
 }
 
 }  // namespace
 
 cudaError_t launch_coarse(const CoarseLaunch& L, cudaStream_t stream) {
   if (L.n_videos == 0) return cudaSuccess;
-  if (L.total_text > 0) {
-    // groups of 8 text rows per video: at most total_text / 8 + one partial group per video;
-    // CTAs past the last group return at once
-    dim3 g1((L.total_text + 7) / 8 + L.n_videos, L.hq);
-    coarse_rows_kernel<<<g1, 256, 0, stream>>>(L);
-    cudaError_t e = cudaGetLastError();
+  cudaError_t e = cudaSuccess;
+  if (L.total_text > 0 && L.max_blocks > 0) {
+    e = L.head_dim == 128 ? launch_rows<128>(L, stream) : launch_rows<64>(L, stream);
     if (e != cudaSuccess) return e;
   }
-  if (L.max_frames > 0) {
-    dim3 g2((L.max_frames + 127) / 128, L.hq, L.n_videos);
-    coarse_map_kernel<<<g2, 128, 0, stream>>>(L);
-    cudaError_t e = cudaGetLastError();
+  if (L.total_vis > 0) {
+    dim3 g((L.total_vis / L.block) / 32 + L.n_videos, L.hq);
+    coarse_map_kernel<<<g, kMapWarps * 32, 0, stream>>>(L);
+    e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
-  dim3 g3(std::max(1, (L.max_frames + 127) / 128), L.n_videos);
-  coarse_finalize_kernel<<<g3, 128, 0, stream>>>(L);
+  const int head_blocks = (L.hq + kFinalWarps - 1) / kFinalWarps;
+  const int aqf_blocks = (L.total_frames + kFinalWarps * 32 - 1) / (kFinalWarps * 32);
+  coarse_finalize_kernel<<<L.n_videos * head_blocks + aqf_blocks, kFinalWarps * 32, 0, stream>>>(L, head_blocks);
   return cudaGetLastError();
 }
 

@@ -860,7 +860,7 @@ int evisel_topp_mask(const evisel_probe_args* a, int32_t block, float tau_p, uin
   // Videos, their blocks and row tiles (128 rows: the visual rows, then the text rows).
   std::vector<ToppVideo> vids;
   std::vector<ToppRowTile> tiles;
-  int blk_off = 0, row_tile0 = 0, max_blocks = 0, max_vis_tiles = 0;
+  int blk_off = 0, row_tile0 = 0, max_blocks = 0, max_vis_tiles = 0, text_off = 0, vis_off = 0;
   for (int b = 0; b < a->num_videos; ++b) {
     ToppVideo v{};
     v.start = a->cu_seqlens_h[b];
@@ -868,6 +868,10 @@ int evisel_topp_mask(const evisel_probe_args* a, int32_t block, float tau_p, uin
     v.n_text = a->cu_seqlens_h[b + 1] - v.start - v.n_vis;
     v.blk_off = blk_off;
     v.row_tile0 = row_tile0;
+    v.text_off = text_off;
+    v.vis_off = vis_off;
+    text_off += v.n_text;
+    vis_off += v.n_vis;
     const int nb = v.n_vis / block + (v.n_text + block - 1) / block;
     blk_off += nb;
     max_blocks = std::max(max_blocks, nb);
@@ -979,23 +983,20 @@ int evisel_coarse_evidence(const evisel_probe_args* a, evisel_ws* ws, int32_t bl
     return fail(EVISEL_EINVAL, "args / block do not match the evisel_topp_mask call on this workspace");
   if (a->num_videos == 0) return EVISEL_OK;
   const int npf = a->tokens_per_frame;
-  std::vector<int> text_off(1, 0), vis_off(1, 0), frame_off(1, 0);
-  int max_frames = 0;
+  int total_text = 0, total_vis = 0, total_frames = 0, max_blocks = 0;
   for (int b = 0; b < a->num_videos; ++b) {
     const int nv = a->n_vis_h[b], nt = a->cu_seqlens_h[b + 1] - a->cu_seqlens_h[b] - nv;
-    text_off.push_back(text_off.back() + nt);
-    vis_off.push_back(vis_off.back() + nv);
-    frame_off.push_back(frame_off.back() + nv / npf);
-    max_frames = std::max(max_frames, nv / npf);
+    total_text += nt;
+    total_vis += nv;
+    total_frames += nv / npf;
+    max_blocks = std::max(max_blocks, nv / block + (nt + block - 1) / block);
   }
-  const int total_text = text_off.back();
-  if ((vis_off.back() > 0 && (!tok || !frame)) || !head || (frame_off.back() > 0 && !aqf) || !keep || !a->q || !a->k)
+  if ((total_vis > 0 && (!tok || !frame)) || !head || (total_frames > 0 && !aqf) || !keep || !a->q || !a->k)
     return fail(EVISEL_EINVAL, "an output map, keep, q or k is NULL");
   const int pitch = ws->topp_n_words * 32;
-  const size_t ints = align_up(3 * (a->num_videos + 1) * sizeof(int), 256);
   const size_t gbytes = align_up(static_cast<size_t>(a->hq) * total_text * pitch * sizeof(float), 256);
   const size_t mz = align_up(static_cast<size_t>(a->hq) * total_text * sizeof(float), 256);
-  const size_t need = ints + gbytes + 2 * mz;
+  const size_t need = gbytes + 2 * mz;
   cudaStream_t stream = static_cast<cudaStream_t>(stream_ptr);
   if (need > ws->coarse_bytes) {
     cudaStreamSynchronize(ws->last_stream);
@@ -1009,26 +1010,16 @@ int evisel_coarse_evidence(const evisel_probe_args* a, evisel_ws* ws, int32_t bl
     }
     ws->coarse_bytes = need;
   }
-  std::vector<int> offs;
-  offs.insert(offs.end(), text_off.begin(), text_off.end());
-  offs.insert(offs.end(), vis_off.begin(), vis_off.end());
-  offs.insert(offs.end(), frame_off.begin(), frame_off.end());
   char* d = static_cast<char*>(ws->coarse_buf);
-  cudaError_t e = cudaMemcpyAsync(d, offs.data(), offs.size() * sizeof(int), cudaMemcpyHostToDevice, stream);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(stream);   // the host vector goes out of scope
-  if (e != cudaSuccess) return cuda_fail(e, "coarse-map offsets");
   CoarseLaunch L{};
   L.q = a->q;
   L.k = a->k;
   L.kbar = static_cast<char*>(ws->topp_buf) + ws->topp_kbar_off;
   L.vids = static_cast<const ToppVideo*>(ws->topp_buf);
-  L.text_off = reinterpret_cast<const int*>(d);
-  L.vis_off = L.text_off + (a->num_videos + 1);
-  L.frame_off = L.vis_off + (a->num_videos + 1);
   L.keep = keep;
-  L.gbuf = reinterpret_cast<float*>(d + ints);
-  L.row_m = reinterpret_cast<float*>(d + ints + gbytes);
-  L.row_z = reinterpret_cast<float*>(d + ints + gbytes + mz);
+  L.gbuf = reinterpret_cast<float*>(d);
+  L.row_m = reinterpret_cast<float*>(d + gbytes);
+  L.row_z = reinterpret_cast<float*>(d + gbytes + mz);
   L.tok = tok;
   L.frame = frame;
   L.head = head;
@@ -1043,12 +1034,12 @@ int evisel_coarse_evidence(const evisel_probe_args* a, evisel_ws* ws, int32_t bl
   L.head_dim = a->head_dim;
   L.block = block;
   L.tokens_per_frame = npf;
-  L.total_vis = vis_off.back();
-  L.total_frames = frame_off.back();
-  L.max_frames = max_frames;
+  L.total_vis = total_vis;
+  L.total_frames = total_frames;
+  L.max_blocks = max_blocks;
   L.accumulate = accumulate != 0;
   L.scale = a->softmax_scale > 0.f ? a->softmax_scale : 1.0f / std::sqrt(float(a->head_dim));
-  e = launch_coarse(L, stream);
+  cudaError_t e = launch_coarse(L, stream);
   if (e != cudaSuccess) return cuda_fail(e, "coarse-map launch");
   ws->last_stream = stream;
   return EVISEL_OK;

@@ -198,7 +198,9 @@ struct ToppVideo {
   int32_t n_vis, n_text;
   int32_t blk_off;    // global index of its first block (k_bar rows)
   int32_t row_tile0;  // global index of its first visual row tile of the attention's tiling
-  int32_t pad0, pad1, pad2;
+  int32_t text_off;   // its first text row, text rows of all videos back to back
+  int32_t vis_off;    // its first visual token, visual tokens of all videos back to back
+  int32_t pad0;
 };
 static_assert(sizeof(ToppVideo) == 32, "ToppVideo is 32 bytes");
 
@@ -236,9 +238,6 @@ struct CoarseLaunch {
   const void* k;                    // bf16 [N, hkv, d]
   const void* kbar;                 // bf16 [blocks, hkv, d] (from the builder)
   const ToppVideo* vids;
-  const int* text_off;              // [videos + 1] first text row of each video (text rows back to back)
-  const int* vis_off;               // [videos + 1] column offsets of the token map
-  const int* frame_off;             // [videos + 1] column offsets of the frame map
   const uint32_t* keep;             // [hq, n_words, N]
   float* gbuf;                      // [hq, total_text, pitch] block affinities of the text rows
   float* row_m;                     // [hq, total_text]
@@ -248,7 +247,7 @@ struct CoarseLaunch {
   float* head;
   float* aqf;
   int n_videos, total_text, pitch, n_words, n_tok, hq, hkv, head_dim, block, tokens_per_frame;
-  int total_vis, total_frames, max_frames, accumulate;
+  int total_vis, total_frames, max_blocks, accumulate;
   float scale;
 };
 
