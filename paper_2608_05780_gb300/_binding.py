@@ -9,6 +9,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+import struct
 
 import numpy as np
 
@@ -52,6 +53,11 @@ class ProbeArgs(ctypes.Structure):
     ]
 
 
+# ProbeArgs as one pack (native alignment, the field order above): filling the
+# struct field by field costs several times as much as the call it describes.
+_PACK = struct.Struct("@iPPiiiiifPPPPPPPiiPii")
+assert _PACK.size == ctypes.sizeof(ProbeArgs)
+
 EXPORTS = ["evisel_probe_attention", "evisel_evidence_reduce", "evisel_free", "evisel_status",
            "evisel_strerror", "evisel_last_error", "evisel_workspace_bytes", "evisel_build_id"]
 
@@ -67,7 +73,8 @@ def load(path: str = LIB_PATH):
         raise RuntimeError(f"libevisel.so is not built ({path}); run paper_2608_05780_gb300.build.build()")
     lib = ctypes.CDLL(path)
     vp, i32 = ctypes.c_void_p, ctypes.c_int
-    lib.evisel_probe_attention.argtypes = [ctypes.POINTER(ProbeArgs), vp, ctypes.POINTER(vp)]
+    args_p = vp                 # a ProbeArgs by reference
+    lib.evisel_probe_attention.argtypes = [args_p, vp, ctypes.POINTER(vp)]
     lib.evisel_probe_attention.restype = i32
     lib.evisel_evidence_reduce.argtypes = [vp, vp, vp, vp, vp, i32, vp]
     lib.evisel_evidence_reduce.restype = i32
@@ -83,16 +90,16 @@ def load(path: str = LIB_PATH):
     lib.evisel_workspace_bytes.restype = ctypes.c_int64
     lib.evisel_build_id.argtypes = []
     lib.evisel_build_id.restype = ctypes.c_char_p
-    lib.evisel_probe_evidence_noalloc.argtypes = [ctypes.POINTER(ProbeArgs), vp, vp, vp, vp, i32, vp,
+    lib.evisel_probe_evidence_noalloc.argtypes = [args_p, vp, vp, vp, vp, i32, vp,
                                                   ctypes.POINTER(ctypes.c_int)]
     lib.evisel_probe_evidence_noalloc.restype = i32
-    lib.evisel_intra_frame_evidence.argtypes = [ctypes.POINTER(ProbeArgs), vp, vp, i32, vp]
+    lib.evisel_intra_frame_evidence.argtypes = [args_p, vp, vp, i32, vp]
     lib.evisel_intra_frame_evidence.restype = i32
-    lib.evisel_cross_frame_evidence.argtypes = [ctypes.POINTER(ProbeArgs), vp, vp, vp, i32, vp]
+    lib.evisel_cross_frame_evidence.argtypes = [args_p, vp, vp, vp, i32, vp]
     lib.evisel_cross_frame_evidence.restype = i32
-    lib.evisel_topp_mask.argtypes = [ctypes.POINTER(ProbeArgs), i32, ctypes.c_float, vp, vp, vp, ctypes.POINTER(vp)]
+    lib.evisel_topp_mask.argtypes = [args_p, i32, ctypes.c_float, vp, vp, vp, ctypes.POINTER(vp)]
     lib.evisel_topp_mask.restype = i32
-    lib.evisel_coarse_evidence.argtypes = [ctypes.POINTER(ProbeArgs), vp, i32, vp, vp, vp, vp, vp, i32, vp]
+    lib.evisel_coarse_evidence.argtypes = [args_p, vp, i32, vp, vp, vp, vp, vp, i32, vp]
     lib.evisel_coarse_evidence.restype = i32
     lib.evisel_selftest_wait.argtypes = [i32, i32, vp, ctypes.POINTER(ctypes.c_int)]
     lib.evisel_selftest_wait.restype = i32
@@ -105,15 +112,29 @@ def _check(rc):
         raise EviselError(rc, _lib.evisel_last_error().decode())
 
 
+_I32 = np.dtype(np.int32)
+
+
 def _i32(a):
-    arr = np.ascontiguousarray(np.asarray(a, dtype=np.int32))
-    return arr, arr.ctypes.data_as(ctypes.POINTER(ctypes.c_int32))
+    """``a`` as a contiguous int32 array (itself where it is one), and its address."""
+    if not (type(a) is np.ndarray and a.dtype == _I32 and a.flags.c_contiguous):
+        a = np.ascontiguousarray(np.asarray(a, dtype=np.int32))
+    return a, a.__array_interface__["data"][0]
+
+
+_raw_stream = None      # torch's own lookup of the current stream's handle, where it has one
 
 
 def _stream_handle(stream):
+    global _raw_stream
+    if stream is not None:
+        return stream.cuda_stream
     import torch
-    s = torch.cuda.current_stream() if stream is None else stream
-    return ctypes.c_void_p(s.cuda_stream)
+    if _raw_stream is None:
+        _raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", False)
+    if _raw_stream and torch.cuda.is_initialized():
+        return _raw_stream(torch.cuda.current_device())
+    return torch.cuda.current_stream().cuda_stream
 
 
 class Workspace:
@@ -145,26 +166,13 @@ def make_args(q, k, v, cu_seqlens, n_vis, tokens_per_frame, tile, row_ptr, col_i
     nv, nv_p = _i32(n_vis)
     rp, rp_p = _i32(row_ptr)
     ci, ci_p = _i32(col_idx if len(col_idx) else np.zeros(1, np.int32))
-    a = ProbeArgs()
-    a.num_videos = len(nv)
-    a.cu_seqlens_h = cu_p
-    a.n_vis_h = nv_p
-    a.tokens_per_frame = int(tokens_per_frame)
-    a.hq = int(q.shape[1])
-    a.hkv = int(k.shape[1])
-    a.head_dim = int(q.shape[2])
-    a.tile = int(tile)
-    a.softmax_scale = float(softmax_scale)
-    a.q, a.k, a.v = q.data_ptr(), k.data_ptr(), v.data_ptr()
-    a.mask_row_ptr_h = rp_p
-    a.mask_col_idx_h = ci_p
-    a.o, a.lse = o.data_ptr(), lse.data_ptr()
-    a.cross_frame = int(bool(cross_frame))
-    a.text_evidence = int(bool(text_evidence))
-    if keep is not None:
-        a.keep = keep.data_ptr()
-        a.keep_words = int(keep.shape[1])
-        a.keep_block = int(keep_block)
+    _, hq, d = q.shape
+    a = ProbeArgs.from_buffer_copy(_PACK.pack(
+        len(nv), cu_p, nv_p, int(tokens_per_frame), int(hq), int(k.shape[1]), int(d), int(tile),
+        ctypes.c_float(softmax_scale).value,
+        q.data_ptr(), k.data_ptr(), v.data_ptr(), rp_p, ci_p, o.data_ptr(), lse.data_ptr(), int(bool(cross_frame)),
+        int(bool(text_evidence)), 0 if keep is None else keep.data_ptr(), 0 if keep is None else int(keep.shape[1]),
+        0 if keep is None else int(keep_block)))
     return a, (cu, nv, rp, ci)
 
 
@@ -207,17 +215,19 @@ def evisel_evidence_reduce(ws, hq, n_vis, tokens_per_frame, num_videos, tok=None
     """
     import torch
     lib = load()
-    total_vis = int(np.sum(n_vis))
-    total_frames = total_vis // int(tokens_per_frame)
-    f32 = dict(dtype=torch.float32, device=device)
-    if tok is None:
-        tok = torch.zeros((hq, total_vis), **f32)
-    if frame is None:
-        frame = torch.zeros((hq, total_frames), **f32)
-    if head is None:
-        head = torch.zeros((num_videos, hq), **f32)
-    if aqf is None:
-        aqf = torch.zeros((total_frames,), **f32)
+    if tok is None or frame is None or head is None or aqf is None:
+        # The call overwrites every entry unless it accumulates (head and A_qf always).
+        total_vis = sum(map(int, n_vis))
+        total_frames = total_vis // int(tokens_per_frame)
+        new = torch.zeros if accumulate else torch.empty
+        if tok is None:
+            tok = new((hq, total_vis), dtype=torch.float32, device=device)
+        if frame is None:
+            frame = new((hq, total_frames), dtype=torch.float32, device=device)
+        if head is None:
+            head = torch.zeros((num_videos, hq), dtype=torch.float32, device=device)
+        if aqf is None:
+            aqf = new((total_frames,), dtype=torch.float32, device=device)
     _check(lib.evisel_evidence_reduce(ws.ptr, tok.data_ptr(), frame.data_ptr(), head.data_ptr(),
                                       aqf.data_ptr(), int(bool(accumulate)), _stream_handle(stream)))
     return tok, frame, head, aqf
@@ -344,20 +354,13 @@ def evisel_topp_mask(q, k, cu_seqlens, n_vis, tokens_per_frame, tile, block, tau
 
 def tile_union_to_csr(tile_union, n_vis, tile):
     """Host CSR (row_ptr, col_idx) of a tile union from evisel_topp_mask."""
-    bits = tile_union.cpu().numpy().view(np.uint32)
-    row_ptr, cols = [0], []
-    r = 0
-    for nv in np.asarray(n_vis, dtype=np.int64):
-        for _ in range(-(-int(nv) // int(tile))):
-            for w, word in enumerate(bits[r]):
-                word = int(word)
-                while word:
-                    low = word & -word
-                    cols.append(w * 32 + low.bit_length() - 1)
-                    word ^= low
-            row_ptr.append(len(cols))
-            r += 1
-    return np.array(row_ptr, np.int32), np.array(cols, np.int32)
+    words = np.ascontiguousarray(tile_union.cpu().numpy()).view(np.uint32)
+    rows = int(sum(-(-int(nv) // int(tile)) for nv in np.asarray(n_vis, dtype=np.int64)))
+    bits = np.unpackbits(words[:rows].astype("<u4", copy=False).view(np.uint8), axis=1, bitorder="little")
+    row, col = np.nonzero(bits)                 # row by row, ascending within a row
+    row_ptr = np.zeros(rows + 1, np.int32)
+    np.cumsum(np.bincount(row, minlength=rows), out=row_ptr[1:])
+    return row_ptr, col.astype(np.int32)
 
 
 def evisel_coarse_evidence(q, k, cu_seqlens, n_vis, tokens_per_frame, tile, block, keep, ws, tok=None, frame=None,

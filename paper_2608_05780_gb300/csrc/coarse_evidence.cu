@@ -27,8 +27,8 @@
 // row's own keys (a load and a warp sum per key), over the text rows of a frame
 // in one thread and over a head's frames in one thread took 64, 40 and 15 us on
 // 16,388 tokens (28 heads, 100 text rows, B = 32); here the logits, rows, map and
-//   finalize kernels take 22, 14, 9 and 3 us, the call 137 -> 56 us (its per-video
-//   offsets now come with the builder's upload: no copy, no synchronisation).
+// finalize kernels take 22, 14, 9 and 3 us, the call 137 -> 56 us (its per-video
+// offsets now come with the builder's upload: no copy, no synchronisation).
 #include <cstdint>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>

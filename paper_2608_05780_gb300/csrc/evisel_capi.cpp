@@ -98,7 +98,8 @@ struct Plan {
   int max_frames = 0;
 };
 
-int validate(const evisel_probe_args* a) {
+// Everything but the mask's contents.
+int validate_shape(const evisel_probe_args* a) {
   if (!a) return fail(EVISEL_EINVAL, "args is NULL");
   if (a->num_videos < 0) return fail(EVISEL_EINVAL, "num_videos < 0");
   if (a->num_videos > 0 && (!a->cu_seqlens_h || !a->n_vis_h))
@@ -152,7 +153,18 @@ int validate(const evisel_probe_args* a) {
       return fail(EVISEL_EINVAL, "device pointers must be 16-byte aligned");
   }
   if (rows > 0 && (!a->mask_row_ptr_h || !a->mask_col_idx_h)) return fail(EVISEL_EINVAL, "mask is NULL");
-  if (rows > 0) {
+  return EVISEL_OK;
+}
+
+int64_t mask_rows(const evisel_probe_args* a) {
+  int64_t rows = 0;
+  for (int b = 0; b < a->num_videos; ++b) rows += (a->n_vis_h[b] + a->tile - 1) / a->tile;
+  return rows;
+}
+
+// The mask's contents, after validate_shape.
+int validate_mask(const evisel_probe_args* a) {
+  if (mask_rows(a) > 0) {
     const int32_t* rp = a->mask_row_ptr_h;
     const int32_t* ci = a->mask_col_idx_h;
     if (rp[0] != 0) return fail(EVISEL_EMASK, "mask row_ptr[0] must be 0");
@@ -176,6 +188,11 @@ int validate(const evisel_probe_args* a) {
     }
   }
   return EVISEL_OK;
+}
+
+int validate(const evisel_probe_args* a) {
+  const int rc = validate_shape(a);
+  return rc != EVISEL_OK ? rc : validate_mask(a);
 }
 
 void build_plan(const evisel_probe_args* a, Plan& P) {
@@ -430,13 +447,36 @@ std::vector<int32_t> plan_key(const evisel_probe_args* a) {
                             a->text_evidence, a->keep != nullptr};   // the item order differs with keep bits
   for (int b = 0; b <= a->num_videos && a->num_videos > 0; ++b) k.push_back(a->cu_seqlens_h[b]);
   for (int b = 0; b < a->num_videos; ++b) k.push_back(a->n_vis_h[b]);
-  int64_t rows = 0;
-  for (int b = 0; b < a->num_videos; ++b) rows += (a->n_vis_h[b] + a->tile - 1) / a->tile;
+  const int64_t rows = mask_rows(a);
   if (rows > 0) {
     k.insert(k.end(), a->mask_row_ptr_h, a->mask_row_ptr_h + rows + 1);
     k.insert(k.end(), a->mask_col_idx_h, a->mask_col_idx_h + a->mask_row_ptr_h[rows]);
   }
   return k;
+}
+
+// Whether plan_key(a) == key, by value and without building it: the plan that
+// the key was made for (and its checked mask) then stands for these arguments.
+// Needs validate_shape.
+bool key_matches(const evisel_probe_args* a, const std::vector<int32_t>& key) {
+  const int32_t head[] = {a->num_videos, a->tokens_per_frame, a->hq, a->hkv, a->head_dim, a->tile, a->cross_frame,
+                          a->text_evidence, a->keep != nullptr};
+  const int32_t* k = key.data();
+  size_t left = key.size();
+  auto same = [&](const int32_t* p, size_t n) {
+    if (n > left || (n > 0 && std::memcmp(p, k, n * sizeof(int32_t)) != 0)) return false;
+    k += n;
+    left -= n;
+    return true;
+  };
+  if (!same(head, sizeof(head) / sizeof(head[0]))) return false;
+  if (a->num_videos > 0 && (!same(a->cu_seqlens_h, a->num_videos + 1) || !same(a->n_vis_h, a->num_videos))) return false;
+  const int64_t rows = mask_rows(a);
+  if (rows > 0) {
+    if (!same(a->mask_row_ptr_h, rows + 1)) return false;      // row_ptr[rows] is then the checked one
+    if (!same(a->mask_col_idx_h, a->mask_row_ptr_h[rows])) return false;
+  }
+  return left == 0;
 }
 
 template <typename T>
@@ -587,7 +627,11 @@ int evisel_probe_attention(const evisel_probe_args* args, void* stream_ptr, evis
   const NvtxRange nvtx_range("evisel_probe_attention");
   g_last_error.clear();
   if (!ws_inout) return fail(EVISEL_EINVAL, "ws_inout is NULL");
-  int rc = validate(args);
+  int rc = validate_shape(args);
+  if (rc != EVISEL_OK) return rc;
+  // The same description as the plan at hand (by value): its mask is checked already.
+  const bool planned = *ws_inout && (*ws_inout)->have_plan && key_matches(args, (*ws_inout)->key);
+  if (!planned) rc = validate_mask(args);
   if (rc != EVISEL_OK) return rc;
   cudaStream_t stream = static_cast<cudaStream_t>(stream_ptr);
   if (!*ws_inout) {
@@ -599,8 +643,8 @@ int evisel_probe_attention(const evisel_probe_args* args, void* stream_ptr, evis
   cudaGetDevice(&dev);
   if (dev != ws->device) return fail(EVISEL_EINVAL, "workspace belongs to another device");
 
-  std::vector<int32_t> key = plan_key(args);
-  if (!ws->have_plan || key != ws->key) {
+  if (!planned) {
+    std::vector<int32_t> key = plan_key(args);
     ws->plan = Plan();
     build_plan(args, ws->plan);
     ws->have_plan = false;
@@ -728,7 +772,8 @@ int evisel_intra_frame_evidence(const evisel_probe_args* args, const evisel_ws* 
   g_last_error.clear();
   evisel_ws* ws = const_cast<evisel_ws*>(ws_c);
   if (!ws) return fail(EVISEL_EINVAL, "workspace is NULL");
-  int rc = validate(args);
+  int rc = validate_shape(args);
+  if (rc == EVISEL_OK && !(ws->have_plan && key_matches(args, ws->key))) rc = validate_mask(args);
   if (rc != EVISEL_OK) return rc;
   if (!ws->probed || !ws->have_plan) return fail(EVISEL_ESTATE, "no probe has run on this workspace");
   if (ws->probe_keep) return fail(EVISEL_EUNSUPPORTED, "the probe ran with per-row block masks");
@@ -777,13 +822,15 @@ int evisel_cross_frame_evidence(const evisel_probe_args* args, evisel_ws* ws, fl
   const NvtxRange nvtx_range("evisel_cross_frame_evidence");
   g_last_error.clear();
   if (!ws) return fail(EVISEL_EINVAL, "workspace is NULL");
-  int rc = validate(args);
+  int rc = validate_shape(args);
+  const bool planned = rc == EVISEL_OK && ws->have_plan && key_matches(args, ws->key);
+  if (rc == EVISEL_OK && !planned) rc = validate_mask(args);
   if (rc != EVISEL_OK) return rc;
   if (!ws->probed || !ws->have_plan) return fail(EVISEL_ESTATE, "no probe has run on this workspace");
   const Plan& P = ws->plan;
   if (!P.cross_frame) return fail(EVISEL_ESTATE, "the probe on this workspace ran without cross_frame");
   if (ws->probe_keep) return fail(EVISEL_EUNSUPPORTED, "the probe ran with per-row block masks");
-  if (static_cast<int>(P.videos.size()) != args->num_videos || plan_key(args) != ws->key)
+  if (static_cast<int>(P.videos.size()) != args->num_videos || !planned)
     return fail(EVISEL_EINVAL, "args do not match the probe that ran on this workspace");
   if (P.aff_floats > 0 && !aff) return fail(EVISEL_EINVAL, "aff is NULL");
   cudaStream_t stream = static_cast<cudaStream_t>(stream_ptr);

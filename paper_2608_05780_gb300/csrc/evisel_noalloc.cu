@@ -46,7 +46,7 @@ constexpr size_t kScratchBytes = static_cast<size_t>(EVISEL_NOALLOC_SCRATCH_BYTE
 constexpr size_t kStageBytes = size_t(4) << 20;     // largest plan (work list, kv lists, tables)
 constexpr int kMaxDevices = 64;
 
-alignas(256) unsigned char g_stage[kStageBytes];    // host staging of the plan
+alignas(256) unsigned char g_stage[kStageBytes + 256];   // host staging of the status word and the plan
 std::mutex g_mutex;
 void* g_scratch_ptr[kMaxDevices] = {};
 
@@ -240,18 +240,17 @@ extern "C" int evisel_probe_evidence_noalloc(const evisel_probe_args* args, floa
   unsigned char* base = static_cast<unsigned char*>(g_scratch_ptr[dev]);
   cudaStream_t stream = static_cast<cudaStream_t>(stream_ptr);
 
-  Out out{reinterpret_cast<WorkItem*>(g_stage + (o_items - 256)), reinterpret_cast<KvTile*>(g_stage + (o_kv - 256)),
-          reinterpret_cast<VideoInfo*>(g_stage + (o_videos - 256)),
-          reinterpret_cast<CombineGroup*>(g_stage + (o_groups - 256)),
-          reinterpret_cast<EvChunk*>(g_stage + (o_chunks - 256))};
+  Out out{reinterpret_cast<WorkItem*>(g_stage + o_items), reinterpret_cast<KvTile*>(g_stage + o_kv),
+          reinterpret_cast<VideoInfo*>(g_stage + o_videos),
+          reinterpret_cast<CombineGroup*>(g_stage + o_groups),
+          reinterpret_cast<EvChunk*>(g_stage + o_chunks)};
   make_plan(args, c, &out);
 
-  // The status word must start at zero; the rest is fully written before it is read.
-  e = cudaMemsetAsync(base, 0, sizeof(int), stream);
-  // Pageable source: the copy is staged before cudaMemcpyAsync returns, so g_stage
-  // may be rewritten by the next call.
-  if (e == cudaSuccess && meta_end > 256)
-    e = cudaMemcpyAsync(base + 256, g_stage, meta_end - 256, cudaMemcpyHostToDevice, stream);
+  // The status word must start at zero and goes with the plan; the rest is fully
+  // written before it is read. Pageable source: the copy is staged before
+  // cudaMemcpyAsync returns, so g_stage may be rewritten by the next call.
+  std::memset(g_stage, 0, sizeof(int));
+  e = cudaMemcpyAsync(base, g_stage, meta_end, cudaMemcpyHostToDevice, stream);
   if (e != cudaSuccess) {
     cudaGetLastError();
     return set_last_error(EVISEL_ECUDA, (std::string("plan upload: ") + cudaGetErrorString(e)).c_str());
@@ -355,8 +354,8 @@ extern "C" int evisel_probe_evidence_noalloc(const evisel_probe_args* args, floa
     }
   }
   if (device_status) {
-    e = cudaStreamSynchronize(stream);
-    if (e == cudaSuccess) e = cudaMemcpy(device_status, base, sizeof(int), cudaMemcpyDeviceToHost);
+    e = cudaMemcpyAsync(device_status, base, sizeof(int), cudaMemcpyDeviceToHost, stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
     if (e != cudaSuccess) {
       cudaGetLastError();
       return set_last_error(EVISEL_ECUDA, (std::string("status read: ") + cudaGetErrorString(e)).c_str());
