@@ -35,7 +35,7 @@
 //   digit value in register bins; then every block whose key is below the
 //   boundary key is kept and, at the boundary key, blocks in id order while the
 //   mass before them is below tau_p Z.
-// topp_union_kernel: per (visual row tile, 1,024 blocks) the OR of the rows'
+// topp_union_kernel: per (visual row tile, 512 blocks) the OR of the rows'
 //   bits over the heads, folded into key tiles, as its attention row tiles'
 //   union words.
 // Every wait is bounded; a timeout records EVISEL_ETIMEOUT.
@@ -118,6 +118,11 @@ __device__ __forceinline__ void record_failure(volatile int* abort_flag, int* st
   atomicExch(status, kStatusTimeout);
 }
 
+// One CTA per (block, KV head), one thread per dim. A dim's keys are added in
+// token order in fp32 (k_bar's bf16 rounding, and with it the mask, hangs on
+// that order), so the sum stays serial; its loads go out 16 at a time ahead of
+// the adds (four at a time left the kernel at memory latency: 14 us on 24,704
+// tokens of 4 KV heads, this 9.9).
 __global__ void __launch_bounds__(128) kbar_kernel(const __grid_constant__ ToppLaunch L) {
   // blockIdx.x: global block (video blocks back to back), blockIdx.y: KV head.
   const int gb = blockIdx.x, g = blockIdx.y;
@@ -129,11 +134,21 @@ __global__ void __launch_bounds__(128) kbar_kernel(const __grid_constant__ ToppL
   const int nvb = vid.n_vis / L.block;
   const int start = j < nvb ? j * L.block : vid.n_vis + (j - nvb) * L.block;
   const int len = j < nvb ? L.block : min(L.block, vid.n_vis + vid.n_text - start);
-  const __nv_bfloat16* k = static_cast<const __nv_bfloat16*>(L.k);
+  const int stride = L.hkv * L.head_dim;
   for (int e = threadIdx.x; e < L.head_dim; e += blockDim.x) {
+    const unsigned short* k = static_cast<const unsigned short*>(L.k) +
+                              (static_cast<int64_t>(vid.start + start) * L.hkv + g) * L.head_dim + e;
     float s = 0.f;
-    for (int t = 0; t < len; ++t)
-      s += __bfloat162float(k[(static_cast<int64_t>(vid.start + start + t) * L.hkv + g) * L.head_dim + e]);
+    int t = 0;
+    for (; t + 16 <= len; t += 16) {
+      uint32_t x[16];
+#pragma unroll
+      for (int i = 0; i < 16; ++i) x[i] = __ldg(k + static_cast<int64_t>(i) * stride);
+      k += static_cast<int64_t>(16) * stride;
+#pragma unroll
+      for (int i = 0; i < 16; ++i) s += __uint_as_float(x[i] << 16);
+    }
+    for (; t < len; ++t, k += stride) s += __uint_as_float(static_cast<uint32_t>(__ldg(k)) << 16);
     static_cast<__nv_bfloat16*>(L.kbar)[(static_cast<int64_t>(gb) * L.hkv + g) * L.head_dim + e] =
         __float2bfloat16_rn(s / static_cast<float>(len));
   }
@@ -764,32 +779,35 @@ __device__ __forceinline__ uint32_t compress(uint32_t x) {
   }
 }
 
-constexpr int kUnionWords = 32;                  // keep words (1,024 blocks) per union CTA
+constexpr int kUnionWords = 16;                  // keep words (512 blocks) per union CTA
+constexpr int kUnionHeads = 4;                   // threads per row: heads are dealt over them
 
-// blockIdx.x: builder row tile (visual rows), blockIdx.y: a chunk of 32 keep
-// words, i.e. 32 / BPT words of the union. A thread ORs its row's words over
-// the heads (32 independent loads per head), masks them to the visual blocks,
-// folds blocks into key tiles, the warps OR their rows (shuffles, then shared
-// memory), and one thread stores each union word of each attention row tile
-// the CTA covers (one writer per word: no atomics).
+// blockIdx.x: builder row tile (visual rows), blockIdx.y: a chunk of 16 keep
+// words, i.e. 16 / BPT words of the union. Four threads per row OR its words over
+// every fourth head (16 independent loads per head; one thread over all heads
+// and 32 words was bound by latency: 133 us on 24,704 tokens, 28 heads, this 21;
+// 194 and 84 on 65,664), mask them to the visual blocks, fold blocks into key tiles, the warps OR their rows
+// (shuffles, then shared memory), and one thread stores each union word of each
+// attention row tile the CTA covers (one writer per word: no atomics).
 template <int BPT>
-__global__ void __launch_bounds__(128) topp_union_kernel(const __grid_constant__ ToppLaunch L) {
+__global__ void __launch_bounds__(128 * kUnionHeads) topp_union_kernel(const __grid_constant__ ToppLaunch L) {
   constexpr int kTileWords = kUnionWords / BPT;
-  __shared__ uint32_t part[4][kTileWords];
+  __shared__ uint32_t part[4 * kUnionHeads][kTileWords];
   const ToppRowTile rt = L.tiles[blockIdx.x];
   if (rt.text) return;                           // the attention takes tile masks for visual rows only
   const ToppVideo vid = L.vids[rt.video];
   const int nvb = vid.n_vis / L.block;           // visual blocks (visual rows keep no text block)
   const int w0 = blockIdx.y * kUnionWords;
   if (w0 * 32 >= nvb) return;                    // uniform: no visual block in this chunk
-  const int row = threadIdx.x, lane = row & 31, warp = row >> 5;
+  const int row = threadIdx.x & 127, lane = row & 31, warp = threadIdx.x >> 5;   // warp & 3: its rows
   const bool row_ok = row < rt.q_len;
   uint32_t acc[kUnionWords];
 #pragma unroll
   for (int i = 0; i < kUnionWords; ++i) acc[i] = 0u;
   if (row_ok) {
     const uint32_t* kp = L.keep + static_cast<int64_t>(w0) * L.n_tok + rt.q_start + row;
-    for (int h = 0; h < L.hq; ++h) {
+#pragma unroll 2
+    for (int h = threadIdx.x >> 7; h < L.hq; h += kUnionHeads) {
       const uint32_t* kh = kp + static_cast<int64_t>(h) * L.n_words * L.n_tok;
 #pragma unroll
       for (int i = 0; i < kUnionWords; ++i)
@@ -821,7 +839,9 @@ __global__ void __launch_bounds__(128) topp_union_kernel(const __grid_constant__
   const int t = threadIdx.x / kTileWords, j = threadIdx.x % kTileWords;
   if (t < n_at) {
     uint32_t bits = 0u;
-    for (int ww = t * wpt; ww < (t + 1) * wpt; ++ww) bits |= part[ww][j];
+#pragma unroll
+    for (int g = 0; g < kUnionHeads; ++g)
+      for (int ww = t * wpt; ww < (t + 1) * wpt; ++ww) bits |= part[g * 4 + ww][j];
     const int tile_word = w0 / BPT + j;
     if (tile_word < L.n_tile_words)
       L.tile_union[static_cast<int64_t>(vid.row_tile0 + rt.local0 / L.tile + t) * L.n_tile_words + tile_word] = bits;
@@ -857,10 +877,10 @@ cudaError_t launch_topp(const ToppLaunch& L, cudaStream_t stream) {
   if (L.tile_union) {
     dim3 grid(L.n_tiles, (L.n_words + kUnionWords - 1) / kUnionWords);
     const int bpt = L.tile / L.block;
-    if (bpt == 1) topp_union_kernel<1><<<grid, 128, 0, stream>>>(L);
-    else if (bpt == 2) topp_union_kernel<2><<<grid, 128, 0, stream>>>(L);
-    else if (bpt == 4) topp_union_kernel<4><<<grid, 128, 0, stream>>>(L);
-    else if (bpt == 8) topp_union_kernel<8><<<grid, 128, 0, stream>>>(L);
+    if (bpt == 1) topp_union_kernel<1><<<grid, 128 * kUnionHeads, 0, stream>>>(L);
+    else if (bpt == 2) topp_union_kernel<2><<<grid, 128 * kUnionHeads, 0, stream>>>(L);
+    else if (bpt == 4) topp_union_kernel<4><<<grid, 128 * kUnionHeads, 0, stream>>>(L);
+    else if (bpt == 8) topp_union_kernel<8><<<grid, 128 * kUnionHeads, 0, stream>>>(L);
     else return cudaErrorInvalidValue;
     return cudaGetLastError();
   }
