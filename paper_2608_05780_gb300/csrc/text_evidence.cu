@@ -317,8 +317,8 @@ __global__ void __launch_bounds__(kThreads, 1) text_evidence_kernel(const __grid
     // than a load.
     struct Step {
       float lse[kMaxText / 32];
-      uint32_t bits[kKeep ? kMaxText / 32 : 1];    // per row: bit i = the unit's i-th block is kept
-      int rows, buf;
+      uint32_t bits[kKeep ? kMaxText / 32 : 1];    // per row: bit shift + i = the unit's i-th block is kept
+      int shift, rows, buf;
       bool valid;
     };
     int u = blockIdx.x, hh = 0, tt = 0, nh = 0;
@@ -335,16 +335,19 @@ __global__ void __launch_bounds__(kThreads, 1) text_evidence_kernel(const __grid
       s.rows = x.tile_rows;
       s.buf = nh & (nb - 1);
       const float* lse = L.lse + static_cast<int64_t>(x.h0 + hh) * L.n_tok + x.vis_start + x.n_vis;
+      [[maybe_unused]] const uint32_t* words = nullptr;
+      if constexpr (kKeep) {
+        const int blk0 = x.col0 / L.keep_block;    // a multiple of nblk: the unit's blocks share one word
+        s.shift = blk0 & 31;
+        words = L.keep + (static_cast<int64_t>(x.h0 + hh) * L.keep_words + (blk0 >> 5)) * L.n_tok + x.vis_start + x.n_vis;
+      }
 #pragma unroll
       for (int i = 0; i < kMaxText / 32; ++i) {
         const int r = i * 32 + lane, row = tt * x.tile_rows + r;
         const bool in = r < x.tile_rows && row < x.n_text;
         s.lse[i] = in ? __ldg(lse + row) : INFINITY;   // (no branch and no use here: the loads overlap)
         if constexpr (kKeep) {
-          const int blk0 = x.col0 / L.keep_block;  // a multiple of nblk: the blocks share one word
-          s.bits[i] = in ? __ldg(L.keep + (static_cast<int64_t>(x.h0 + hh) * L.keep_words + (blk0 >> 5)) * L.n_tok +
-                                 x.vis_start + x.n_vis + row) >> (blk0 & 31)
-                         : 0u;
+          s.bits[i] = in ? __ldg(words + row) : 0u;
         }
       }
       if (++tt == x.n_tt) {
@@ -368,7 +371,7 @@ __global__ void __launch_bounds__(kThreads, 1) text_evidence_kernel(const __grid
         for (int i = 0; i < kMaxText / 32; ++i)
           if (i * 32 < s.rows) {
             const float v = -1.4426950408889634f * s.lse[i];
-            if constexpr (kKeep) row[i * 32 + lane] = (s.bits[i] >> kb) & 1u ? v : -INFINITY;
+            if constexpr (kKeep) row[i * 32 + lane] = (s.bits[i] >> (s.shift + kb)) & 1u ? v : -INFINITY;
             else row[i * 32 + lane] = v;
           }
       }
