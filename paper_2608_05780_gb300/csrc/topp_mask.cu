@@ -51,7 +51,7 @@ namespace {
 
 constexpr int kRows = 128;
 constexpr int kCols = 128;                       // blocks per chunk
-constexpr int kHeadSlots = 2;                    // heads in flight
+constexpr int kHeadSlots = 4;                    // heads in flight
 constexpr int kRowWarps = 4 * kHeadSlots;        // warp w: rows 32 (w % 4) .. of head slot w / 4
 constexpr int kWarpProducer = kRowWarps;
 constexpr int kWarpMma = kRowWarps + 1;
@@ -72,21 +72,15 @@ struct TpCfg {
   static constexpr int KB = D / 64;
   static constexpr int TILE_BYTES = kRows * D * 2;   // 128 rows (Q) or 128 blocks (k_bar)
   static constexpr int BLOCK = kRows * 128;
-  static constexpr int OFF_Q = 0;                     // the pair's Q tiles (one stage)
+  static constexpr int OFF_Q = 0;                     // the heads' Q tiles (one stage)
   static constexpr int OFF_K = kHeadSlots * TILE_BYTES;   // 2 stages of k_bar chunks
-  // [32][256] fp32 per row thread: the radix path's u of a 32-column group, or
-  // the fast path's list of window blocks (u), with their ids in [32][256] int32.
-  static constexpr int OFF_STASH = OFF_K + 2 * TILE_BYTES;
-  static constexpr int OFF_LIST_ID = OFF_STASH + kListCap * kRows * kHeadSlots * 4;
-  // [256][32] fp32: the collect pass's u of a 32-column group per row thread,
-  // its 16-byte chunks XOR-swizzled by the thread's row % 8.
-  static constexpr int OFF_GROUP_U = OFF_LIST_ID + kListCap * kRows * kHeadSlots * 4;
-  static constexpr int OFF_BAR = OFF_GROUP_U + 32 * kRows * kHeadSlots * 4;
-  static constexpr int B_QF = 0, B_QE = 1, B_KF = 2, B_KE = 4, B_SF = 6, B_SE = 8, B_DRAIN = 10, B_DEC = 11;
-  static constexpr int N_BARS = 12;
+  static constexpr int OFF_BAR = OFF_K + 2 * TILE_BYTES;
+  static constexpr int B_QF = 0, B_QE = 1, B_KF = 2, B_KE = 4, B_SF = 6, B_SE = B_SF + kHeadSlots,
+                       B_DRAIN = B_SE + kHeadSlots, B_DEC = B_DRAIN + 1;
+  static constexpr int N_BARS = B_DEC + 1;
   static constexpr int OFF_MISC = OFF_BAR + N_BARS * 8;   // TMEM address, abort flag, overflowed pairs
   static constexpr int SMEM_BYTES = OFF_MISC + 16 + 1024;
-  static constexpr int TMEM_COLS = 2 * kHeadSlots * kCols;   // 2 buffers x 2 heads
+  static constexpr int TMEM_COLS = kHeadSlots * kCols;   // one S per head
   static_assert(SMEM_BYTES <= 232448, "shared memory budget");
 };
 
@@ -190,6 +184,19 @@ __device__ __forceinline__ void cum_add(float (&cm)[N], const float (&top)[N], f
   }
 }
 
+// r[e] by selects (e differs between lanes): five levels, no memory.
+__device__ __forceinline__ uint32_t pick32(const uint32_t (&r)[32], int e) {
+  uint32_t a[16];
+#pragma unroll
+  for (int i = 0; i < 16; ++i) a[i] = (e & 16) ? r[i + 16] : r[i];
+#pragma unroll
+  for (int w = 8; w >= 1; w >>= 1)
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+      if (i < w) a[i] = (e & w) ? a[i + w] : a[i];
+  return a[0];
+}
+
 template <int D>
 __global__ void __launch_bounds__(kThreads, 1) topp_select_kernel(const __grid_constant__ ToppLaunch L) {
   using C = TpCfg<D>;
@@ -201,9 +208,11 @@ __global__ void __launch_bounds__(kThreads, 1) topp_select_kernel(const __grid_c
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + C::OFF_MISC + 4);
   uint32_t* overflowed = reinterpret_cast<uint32_t*>(smem + C::OFF_MISC + 8);   // bit min(pair, 31)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const ToppRowTile rt = L.tiles[blockIdx.x];
+  // Last row tiles first: a video's later rows see more blocks, so the long CTAs
+  // start first and the short ones fill the end.
+  const ToppRowTile rt = L.tiles[L.n_tiles - 1 - static_cast<int>(blockIdx.x) / L.hkv];
   const ToppVideo vid = L.vids[rt.video];
-  const int g = blockIdx.y;
+  const int g = static_cast<int>(blockIdx.x) % L.hkv;
   const int gq = L.hq / L.hkv;
   const int nvb = vid.n_vis / L.block;
   // Blocks that end before the tile's last row: the chunk range of this tile.
@@ -212,18 +221,26 @@ __global__ void __launch_bounds__(kThreads, 1) topp_select_kernel(const __grid_c
   };
   const int nh_max = n_hist(rt.local0 + rt.q_len - 1);
   const int n_ch = (nh_max + kCols - 1) / kCols;
-  const int n_pairs = (gq + kHeadSlots - 1) / kHeadSlots;
-  // Work: every pair on the fast path (kFastPasses passes over the n_ch chunks),
-  // then, once every row warp has arrived on B_DEC, the pairs whose window
-  // overflowed a row's list on the radix path (kRadixPasses passes). All roles
-  // step through the same chunk sequence; step t uses S buffer t % 2.
-  auto redo = [&](uint32_t mask, int pair) { return ((mask >> min(pair, 31)) & 1u) != 0u; };
+  const int n_jobs = (gq + kHeadSlots - 1) / kHeadSlots;
+  // Work: every job (kHeadSlots heads) on the fast path (kFastPasses passes over
+  // the n_ch chunks), then, once every row warp has arrived on B_DEC, the pairs
+  // of heads whose window overflowed a row's list on the radix path
+  // (kRadixPasses passes). All roles step through the same chunk sequence; a
+  // slot without a head, or whose pair needs no second path, takes no part.
+  auto takes_part = [&](uint32_t mask, int job, int sl) {
+    const int hh = job * kHeadSlots + sl;
+    return hh < gq && ((mask >> min(hh / 2, 31)) & 1u) != 0u;
+  };
+  auto slots_of = [&](uint32_t mask, int job) {
+    uint32_t m = 0u;
+#pragma unroll
+    for (int sl = 0; sl < kHeadSlots; ++sl) m |= takes_part(mask, job, sl) ? 1u << sl : 0u;
+    return m;
+  };
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < C::N_BARS; ++i)
-      ptx::mbar_init(bar(i), (i == C::B_SE || i == C::B_SE + 1) ? kRows * kHeadSlots
-                             : i == C::B_DEC                      ? kRowWarps
-                                                                  : 1u);
+      ptx::mbar_init(bar(i), i >= C::B_SE && i < C::B_SE + kHeadSlots ? kRows : i == C::B_DEC ? kRowWarps : 1u);
     *abort_flag = 0;
     *overflowed = 0u;
     ptx::fence_mbar_init();
@@ -241,17 +258,17 @@ __global__ void __launch_bounds__(kThreads, 1) topp_select_kernel(const __grid_c
     const uint64_t pol = ptx::l2_policy_evict_last();
     uint32_t leader = 0;
     int nq = 0, nk = 0;                          // Q (per pair job) and k_bar loads issued
-    auto job = [&](int pair, int passes) -> bool {
+    auto job = [&](int j, uint32_t slots, int passes) -> bool {
       if (n_ch == 0) return true;                // no block ends before the tile's rows: nothing to load
       if (nq >= 1 && !warp_wait(bar(C::B_QE), (nq - 1) & 1, abort_flag)) return false;
-      const int nheads = min(kHeadSlots, gq - pair * kHeadSlots);
       if (ptx::elect_one(leader)) {
-        ptx::mbar_arrive_expect_tx(bar(C::B_QF), nheads * C::TILE_BYTES);
-        for (int sl = 0; sl < nheads; ++sl) {
+        ptx::mbar_arrive_expect_tx(bar(C::B_QF), __popc(slots) * C::TILE_BYTES);
+        for (int sl = 0; sl < kHeadSlots; ++sl) {
+          if (!((slots >> sl) & 1u)) continue;
 #pragma unroll
           for (int kb = 0; kb < C::KB; ++kb)
             ptx::tma_load_3d(sbase + C::OFF_Q + sl * C::TILE_BYTES + kb * C::BLOCK, &L.tm_q, bar(C::B_QF),
-                             kb * 64, g * gq + pair * kHeadSlots + sl, rt.q_start, pol);
+                             kb * 64, g * gq + j * kHeadSlots + sl, rt.q_start, pol);
         }
       }
       __syncwarp();
@@ -272,14 +289,14 @@ __global__ void __launch_bounds__(kThreads, 1) topp_select_kernel(const __grid_c
       return true;
     };
     bool ok = true;
-    for (int pair = 0; ok && pair < n_pairs; ++pair) ok = job(pair, kFastPasses);
+    for (int j = 0; ok && j < n_jobs; ++j) ok = job(j, slots_of(~0u, j), kFastPasses);
     uint32_t mask = 0u;
     if (ok) {
       ok = warp_wait(bar(C::B_DEC), 0, abort_flag);
       if (ok) mask = *reinterpret_cast<volatile uint32_t*>(overflowed);
     }
-    for (int pair = 0; ok && pair < n_pairs; ++pair)
-      if (redo(mask, pair)) ok = job(pair, kRadixPasses);
+    for (int j = 0; ok && j < n_jobs; ++j)
+      if (const uint32_t slots = slots_of(mask, j)) ok = job(j, slots, kRadixPasses);
     if (!ok && lane == 0) record_failure(abort_flag, L.status);
     // no copy in flight at exit: the last Q and k_bar loads have landed
     const volatile int never = 0;
@@ -291,50 +308,58 @@ __global__ void __launch_bounds__(kThreads, 1) topp_select_kernel(const __grid_c
     uint32_t leader = 0;
     int first_leader = -1, nj = 0, t = 0;
     bool same = true, issued = false;
-    auto job = [&](int pair, int passes) -> bool {
+    uint32_t used = 0u, parity = 0u;             // per slot: S was written before; parity of its next write
+    auto job = [&](uint32_t slots, int passes) -> bool {
       if (n_ch == 0) return true;                // as the producer: no Q, no steps
-      const int nheads = min(kHeadSlots, gq - pair * kHeadSlots);
       for (int s = 0; s < passes * n_ch; ++s, ++t) {
-        const int b = t % 2;
         if ((s == 0 && !warp_wait(bar(C::B_QF), nj & 1, abort_flag)) ||
-            !warp_wait(bar(C::B_KF + t % 2), (t / 2) & 1, abort_flag) ||
-            (t >= 2 && !warp_wait(bar(C::B_SE + b), ((t - 2) / 2) & 1, abort_flag)))
+            !warp_wait(bar(C::B_KF + t % 2), (t / 2) & 1, abort_flag))
           return false;
-        ptx::tc_fence_after();
         const bool me = ptx::elect_one(leader);
         if (first_leader < 0) first_leader = static_cast<int>(leader);
         same = same && static_cast<int>(leader) == first_leader;
-        if (me && same) {
-          const uint32_t kbase = sbase + C::OFF_K + (t % 2) * C::TILE_BYTES;
-          for (int sl = 0; sl < nheads; ++sl) {
+        if (!same) return false;
+        const uint32_t kbase = sbase + C::OFF_K + (t % 2) * C::TILE_BYTES;
+#pragma unroll 1
+        for (int sl = 0; sl < kHeadSlots; ++sl) {
+          const uint32_t bit = 1u << sl;
+          if (!(slots & bit)) continue;
+          // the slot's rows have read the S before (its parity is that of the write before)
+          if ((used & bit) && !warp_wait(bar(C::B_SE + sl), ((parity >> sl) & 1u) ^ 1u, abort_flag)) return false;
+          ptx::tc_fence_after();
+          if (me) {
             const uint32_t qbase = sbase + C::OFF_Q + sl * C::TILE_BYTES;
 #pragma unroll
             for (int kk = 0; kk < D / 16; ++kk) {
               const uint64_t a = ptx::sdesc_sw128(qbase + (kk / 4) * C::BLOCK + (kk % 4) * 32, 16, 1024);
               const uint64_t bd = ptx::sdesc_sw128(kbase + (kk / 4) * C::BLOCK + (kk % 4) * 32, 16, 1024);
-              ptx::mma_ss(tmem + (b * kHeadSlots + sl) * kCols, a, bd, kIdesc, kk > 0 ? 1u : 0u);
+              ptx::mma_ss(tmem + sl * kCols, a, bd, kIdesc, kk > 0 ? 1u : 0u);
             }
+            ptx::mma_commit(bar(C::B_SF + sl));
           }
-          ptx::mma_commit(bar(C::B_SF + b));
+          __syncwarp();
+          issued = true;
+          used |= bit;
+          parity ^= bit;
+        }
+        if (me) {
           ptx::mma_commit(bar(C::B_KE + t % 2));
           if (s == passes * n_ch - 1) ptx::mma_commit(bar(C::B_QE));
         }
         __syncwarp();
-        issued = true;
-        if (!same) return false;
       }
       ++nj;
       return true;
     };
     bool ok = true;
-    for (int pair = 0; ok && pair < n_pairs; ++pair) ok = job(pair, kFastPasses);
+    for (int j = 0; ok && j < n_jobs; ++j) ok = job(slots_of(~0u, j), kFastPasses);
     uint32_t mask = 0u;
     if (ok) {
       ok = warp_wait(bar(C::B_DEC), 0, abort_flag);
       if (ok) mask = *reinterpret_cast<volatile uint32_t*>(overflowed);
     }
-    for (int pair = 0; ok && pair < n_pairs; ++pair)
-      if (redo(mask, pair)) ok = job(pair, kRadixPasses);
+    for (int j = 0; ok && j < n_jobs; ++j)
+      if (const uint32_t slots = slots_of(mask, j)) ok = job(slots, kRadixPasses);
     if (!ok) {
       if (lane == 0) record_failure(abort_flag, L.status);
       if (issued && lane == first_leader) {
@@ -353,13 +378,12 @@ __global__ void __launch_bounds__(kThreads, 1) topp_select_kernel(const __grid_c
     const uint32_t tbase = tmem + (static_cast<uint32_t>((warp % 4) * 32) << 16) + slot * kCols;
     const float sc = L.scale_log2;               // logits in log2 units
     const float nsc = -sc;
-    constexpr int kStash = kRows * kHeadSlots;   // this thread's column: stash[e * kStash]
-    float* stash = reinterpret_cast<float*>(smem + C::OFF_STASH) + slot * kRows + row;
-    int* list_id = reinterpret_cast<int*>(smem + C::OFF_LIST_ID) + slot * kRows + row;
-    float4* group_u = reinterpret_cast<float4*>(smem + C::OFF_GROUP_U) + (slot * kRows + row) * 8;
-    const int swz = row & 7;
+    // The fast path's list of window blocks (u and id), or the radix path's u of
+    // a 32-column group. A few entries per row and pass: thread-local memory.
+    float stash[kListCap];
+    int list_id[kListCap];
     bool ok = true;
-    int t = 0;                                   // chunk steps consumed
+    int t = 0;                                   // chunk steps this slot consumed
 
     // ---- fast path ----
     // Per pair: (0) the largest and smallest S over H_i; with m = max x
@@ -374,10 +398,10 @@ __global__ void __launch_bounds__(kThreads, 1) topp_select_kernel(const __grid_c
     // from the mass below the window: a block is kept while the mass before it
     // is below tau_p Z. A row whose window holds more than kListCap blocks
     // flags the pair for the radix path.
-    for (int pair = 0; pair < n_pairs; ++pair) {
-      const int hh = pair * kHeadSlots + slot;
-      const bool active = hh < gq;               // warp-uniform: an odd group leaves the last slot idle
-      const int h = g * gq + min(hh, gq - 1);
+    for (int job = 0; job < n_jobs; ++job) {
+      const int hh = job * kHeadSlots + slot;
+      if (!takes_part(~0u, job, slot)) continue; // warp-uniform: a ragged group leaves the last slots idle
+      const int h = g * gq + hh;
       uint32_t* keep = L.keep + static_cast<int64_t>(h) * L.n_words * L.n_tok + rt.q_start + row;
       float smax = -INFINITY, smin = INFINITY, m = 0.f, inv_r = 0.f, z = 0.f, target = 0.f, above = 0.f;
       float lo = 0.f, hi = INFINITY;             // the window: keys lo .. hi - 1 (hi = +inf: up to the last key)
@@ -391,9 +415,9 @@ __global__ void __launch_bounds__(kThreads, 1) topp_select_kernel(const __grid_c
           cm[k] = 0.f;
         }
         for (int ch = 0; ch < n_ch; ++ch, ++t) {
-          const int b = t % 2;
-          ok = ok && warp_wait(bar(C::B_SF + b), (t / 2) & 1, abort_flag);
-          if (ok && active && __any_sync(0xffffffffu, nh > ch * kCols)) {   // warp-uniform: tcgen05.ld is collective
+          bool released = false;
+          ok = ok && warp_wait(bar(C::B_SF + slot), t & 1, abort_flag);
+          if (ok && __any_sync(0xffffffffu, nh > ch * kCols)) {   // warp-uniform: tcgen05.ld is collective
             ptx::tc_fence_after();
 #pragma unroll 1
             for (int c0 = 0; c0 < kCols; c0 += 32) {
@@ -401,8 +425,13 @@ __global__ void __launch_bounds__(kThreads, 1) topp_select_kernel(const __grid_c
               // past every row's H_i only the collect pass has words to write
               if (pass < kFastPasses - 1 && !__any_sync(0xffffffffu, jn > 0)) break;
               uint32_t r[32];
-              ptx::tmem_ld32(tbase + b * kHeadSlots * kCols + c0, r);
+              ptx::tmem_ld32(tbase + c0, r);
               ptx::tmem_wait_ld();
+              if (c0 == kCols - 32) {                        // S is read: the next product may be written
+                ptx::tc_fence_before();
+                ptx::mbar_arrive(bar(C::B_SE + slot));
+                released = true;
+              }
               if (pass == 0) {
                 float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
                 float mn[4] = {INFINITY, INFINITY, INFINITY, INFINITY};
@@ -460,7 +489,6 @@ __global__ void __launch_bounds__(kThreads, 1) topp_select_kernel(const __grid_c
                       else fma2_rn(k1, h1, ik, ih, pw, pw, k1, h1);
                     }
                   }
-                  group_u[e4 ^ swz] = make_float4(uu[0], uu[1], uu[2], uu[3]);
                 }
                 const uint32_t valid = jn >= 32 ? 0xffffffffu : jn > 0 ? (1u << jn) - 1u : 0u;
                 uint32_t word = (__float2uint_rz(k0) | (__float2uint_rz(k1) << 16)) & valid;
@@ -469,8 +497,8 @@ __global__ void __launch_bounds__(kThreads, 1) topp_select_kernel(const __grid_c
                   const int e = __ffs(in_win) - 1;
                   in_win &= in_win - 1u;
                   if (count < kListCap) {
-                    stash[count * kStash] = reinterpret_cast<const float*>(group_u + ((e >> 2) ^ swz))[e & 3];
-                    list_id[count * kStash] = ch * kCols + c0 + e;
+                    stash[count] = __fmaf_rn(__uint_as_float(pick32(r, e)), nsc, m);
+                    list_id[count] = ch * kCols + c0 + e;
                   }
                   ++count;
                 }
@@ -482,7 +510,7 @@ __global__ void __launch_bounds__(kThreads, 1) topp_select_kernel(const __grid_c
               }
             }
             ptx::tc_fence_before();
-          } else if (pass == kFastPasses - 1 && row_ok && ok && active) {
+          } else if (pass == kFastPasses - 1 && row_ok && ok) {
             // No column of this chunk is in H_i for the warp: zeros (and the own block).
             for (int wi = 0; wi < 4; ++wi) {
               const int w = ch * 4 + wi;
@@ -490,7 +518,7 @@ __global__ void __launch_bounds__(kThreads, 1) topp_select_kernel(const __grid_c
               keep[static_cast<int64_t>(w) * L.n_tok] = w == nh >> 5 ? 1u << (nh & 31) : 0u;
             }
           }
-          ptx::mbar_arrive(bar(C::B_SE + b));
+          if (!released) ptx::mbar_arrive(bar(C::B_SE + slot));
         }
         if (pass == 0) {
           m = __fmul_ru(smax, sc);               // >= every x of H_i, so u >= 0
@@ -513,9 +541,9 @@ __global__ void __launch_bounds__(kThreads, 1) topp_select_kernel(const __grid_c
           lo = nlo;
         }
       }
-      if (ok && active && row_ok && count > 0) {
+      if (ok && row_ok && count > 0) {
         if (count > kListCap) {
-          atomicOr(overflowed, 1u << min(pair, 31));
+          atomicOr(overflowed, 1u << min(hh / 2, 31));
         } else {
           // The window's last 8 key bits from the list (in id order): two 4-bit
           // digits by cumulative masses, as the passes take theirs; then every
@@ -532,7 +560,7 @@ __global__ void __launch_bounds__(kThreads, 1) topp_select_kernel(const __grid_c
               cm[k] = base;
             }
             for (int i = 0; i < count; ++i) {
-              const float u = stash[i * kStash];
+              const float u = stash[i];
               float unused = 0.f;
               cum_add(cm, top, __fmaf_rz(u, inv_r, kMagic), ptx::ex2(-u), unused);
             }
@@ -551,7 +579,7 @@ __global__ void __launch_bounds__(kThreads, 1) topp_select_kernel(const __grid_c
           const float t_lo = kMagic + lo, t_hi = kMagic + hi;   // the boundary key (up to the last at the top)
           float tie = 0.f;
           for (int i = 0; i < count; ++i) {
-            const float u = stash[i * kStash];
+            const float u = stash[i];
             const float f = __fmaf_rz(u, inv_r, kMagic);
             bool kept = f < t_lo;
             if (f >= t_lo && f < t_hi) {
@@ -559,7 +587,7 @@ __global__ void __launch_bounds__(kThreads, 1) topp_select_kernel(const __grid_c
               tie = __fadd_rn(tie, ptx::ex2(-u));
             }
             if (kept) {
-              const int id = list_id[i * kStash];
+              const int id = list_id[i];
               atomicOr(keep + static_cast<int64_t>(id >> 5) * L.n_tok, 1u << (id & 31));
             }
           }
@@ -567,7 +595,7 @@ __global__ void __launch_bounds__(kThreads, 1) topp_select_kernel(const __grid_c
       }
       __syncwarp();
       // The own block's word when it lies past the chunks of this tile.
-      if (row_ok && ok && active && (nh >> 5) >= n_ch * 4 && (nh >> 5) < L.n_words)
+      if (row_ok && ok && (nh >> 5) >= n_ch * 4 && (nh >> 5) < L.n_words)
         keep[static_cast<int64_t>(nh >> 5) * L.n_tok] = 1u << (nh & 31);
     }
     __syncwarp();
@@ -578,11 +606,9 @@ __global__ void __launch_bounds__(kThreads, 1) topp_select_kernel(const __grid_c
       if (ok) mask = *reinterpret_cast<volatile uint32_t*>(overflowed);
     }
     // ---- radix path, for the pairs some row flagged ----
-    for (int pair = 0; ok && pair < n_pairs; ++pair) {
-      if (!redo(mask, pair)) continue;
-      const int hh = pair * kHeadSlots + slot;
-      const bool active = hh < gq;               // warp-uniform: an odd group leaves the last slot idle
-      const int h = g * gq + min(hh, gq - 1);
+    for (int job = 0; ok && job < n_jobs; ++job) {
+      if (!takes_part(mask, job, slot)) continue;
+      const int h = g * gq + job * kHeadSlots + slot;
       float m = -INFINITY, gmin = INFINITY, z = 0.f;
       float inv_r = 0.f, target = 0.f, above = 0.f, tie = 0.f;
       int wkey = 0;                              // the boundary's key digits found so far
@@ -600,9 +626,8 @@ __global__ void __launch_bounds__(kThreads, 1) topp_select_kernel(const __grid_c
 #pragma unroll
         for (int k = 0; k < kDigBins; ++k) acc[k] = 0.f;
         for (int ch = 0; ch < n_ch; ++ch, ++t) {
-          const int b = t % 2;
-          ok = ok && warp_wait(bar(C::B_SF + b), (t / 2) & 1, abort_flag);
-          if (ok && active && __any_sync(0xffffffffu, nh > ch * kCols)) {   // warp-uniform: tcgen05.ld is collective
+          ok = ok && warp_wait(bar(C::B_SF + slot), t & 1, abort_flag);
+          if (ok && __any_sync(0xffffffffu, nh > ch * kCols)) {   // warp-uniform: tcgen05.ld is collective
             ptx::tc_fence_after();
             // One compact loop per pass (uniform over the warp), 32 columns at a
             // time. x, the key and the weight use non-contracted arithmetic so
@@ -610,7 +635,7 @@ __global__ void __launch_bounds__(kThreads, 1) topp_select_kernel(const __grid_c
 #pragma unroll 1
             for (int c0 = 0; c0 < kCols; c0 += 32) {
               uint32_t r[32];
-              ptx::tmem_ld32(tbase + b * kHeadSlots * kCols + c0, r);
+              ptx::tmem_ld32(tbase + c0, r);
               ptx::tmem_wait_ld();
               const int jn = nh - (ch * kCols + c0);         // columns e < jn are in H_i
               if (pass == 0) {
@@ -650,13 +675,13 @@ __global__ void __launch_bounds__(kThreads, 1) topp_select_kernel(const __grid_c
                   const float v = __fmul_rn(u, inv_r);
                   if (e < jn && v >= lo && v < hi) {
                     in_mask |= 1u << e;
-                    stash[e * kStash] = u;
+                    stash[e] = u;
                   }
                 }
                 while (in_mask != 0u) {
                   const int e = __ffs(in_mask) - 1;
                   in_mask &= in_mask - 1u;
-                  const float u = stash[e * kStash];
+                  const float u = stash[e];
                   const int key = min(kQMax, __float2int_rz(__fmul_rn(u, inv_r)));
                   bin_add<0, 16>(acc, (key >> dshift) & ((1 << width) - 1), ptx::ex2(-u));
                 }
@@ -673,7 +698,7 @@ __global__ void __launch_bounds__(kThreads, 1) topp_select_kernel(const __grid_c
                   word |= (e < jn && v < k0) ? 1u << e : 0u;
                   if (e < jn && v >= k0 && v < k1) {
                     at_mask |= 1u << e;
-                    stash[e * kStash] = u;
+                    stash[e] = u;
                   }
                 }
                 // the boundary key: lower ids first while the mass before them is below the target
@@ -681,7 +706,7 @@ __global__ void __launch_bounds__(kThreads, 1) topp_select_kernel(const __grid_c
                   const int e = __ffs(at_mask) - 1;
                   at_mask &= at_mask - 1u;
                   if (above + tie < target) word |= 1u << e;
-                  tie += ptx::ex2(-stash[e * kStash]);
+                  tie += ptx::ex2(-stash[e]);
                 }
                 __syncwarp();
                 const int w = ch * 4 + (c0 >> 5);
@@ -692,7 +717,7 @@ __global__ void __launch_bounds__(kThreads, 1) topp_select_kernel(const __grid_c
               }
             }
             ptx::tc_fence_before();
-          } else if (pass == kRadixPasses - 1 && row_ok && ok && active) {
+          } else if (pass == kRadixPasses - 1 && row_ok && ok) {
             // No column of this chunk is in H_i for the warp: zeros (and the own block).
             for (int wi = 0; wi < 4; ++wi) {
               const int w = ch * 4 + wi;
@@ -700,7 +725,7 @@ __global__ void __launch_bounds__(kThreads, 1) topp_select_kernel(const __grid_c
               keep[static_cast<int64_t>(w) * L.n_tok] = w == nh >> 5 ? 1u << (nh & 31) : 0u;
             }
           }
-          ptx::mbar_arrive(bar(C::B_SE + b));
+          ptx::mbar_arrive(bar(C::B_SE + slot));
         }
         // Between passes: the key scale, then per digit the boundary value and
         // the mass above it. The boundary is the first digit value whose
@@ -735,7 +760,7 @@ __global__ void __launch_bounds__(kThreads, 1) topp_select_kernel(const __grid_c
         }
       }
       // The own block's word when it lies past the chunks of this tile.
-      if (row_ok && ok && active && (nh >> 5) >= n_ch * 4 && (nh >> 5) < L.n_words)
+      if (row_ok && ok && (nh >> 5) >= n_ch * 4 && (nh >> 5) < L.n_words)
         keep[static_cast<int64_t>(nh >> 5) * L.n_tok] = 1u << (nh & 31);
     }
     if (!ok && row == 0) record_failure(abort_flag, L.status);
@@ -855,8 +880,7 @@ cudaError_t launch_select(const ToppLaunch& L, cudaStream_t stream) {
   static PerDeviceAttr smem_once;
   cudaError_t e = raise_smem_limit(smem_once, reinterpret_cast<const void*>(kern), C::SMEM_BYTES);
   if (e != cudaSuccess) return e;
-  dim3 grid(L.n_tiles, L.hkv);
-  kern<<<grid, kThreads, C::SMEM_BYTES, stream>>>(L);
+  kern<<<static_cast<unsigned>(L.n_tiles) * L.hkv, kThreads, C::SMEM_BYTES, stream>>>(L);
   return cudaGetLastError();
 }
 
