@@ -11,14 +11,18 @@
 //
 // kbar_kernel: one CTA per (block, KV head): the block's mean key in fp32,
 //   stored as bf16 (the tensor cores' input type).
-// topp_select_kernel: one CTA per (128-row tile of a video, KV group), 320
-//   threads (warp 8 TMA, warp 9 MMA; warps 0-7 one row each, of head slot
-//   warp / 4). The heads of the group go in pairs: S = Q_h k_bar^T for both
-//   heads of a pair, in chunks of 128 blocks (tcgen05, both products from one
-//   k_bar chunk, TMEM 2 buffers x 2 heads), recomputed for every pass over the
-//   chunks. A block's key is q = floor((max - x) 2^14 / (max - min)) over H_i
-//   (0 = the largest logit); blocks are ordered by key, ties by id.
-//   Fast path (every pair), four passes:
+// topp_select_kernel: one CTA per (128-row tile of a video, KV group), 576
+//   threads (warp 16 TMA, warp 17 MMA; warps 0-15 one row each, of head slot
+//   warp / 4). Four heads of the group go at a time: S = Q_h k_bar^T in chunks
+//   of 128 blocks (tcgen05, the products of all slots from one k_bar chunk, one
+//   TMEM tile per slot, given back when its last columns are in registers),
+//   recomputed for every pass over the chunks. Bound by the digit passes' FMA
+//   pipe and issue (60% of the issue slots, FMA pipe 50%): with two heads at a
+//   time, two row warps per scheduler, a mask of 65,664 tokens in blocks of 64
+//   took 2.5 ms, with four 2.0. A block's key is
+//   q = floor((max - x) 2^14 / (max - min)) over H_i (0 = the largest logit);
+//   blocks are ordered by key, ties by id.
+//   Fast path (every head), four passes:
 //     0     the row's max and min logit over H_i;
 //     1, 2  two 3-bit digits of the boundary key: per digit value, the mass of
 //           the blocks whose key lies below its top (a saturated difference of
@@ -257,7 +261,7 @@ __global__ void __launch_bounds__(kThreads, 1) topp_select_kernel(const __grid_c
   if (warp == kWarpProducer) {
     const uint64_t pol = ptx::l2_policy_evict_last();
     uint32_t leader = 0;
-    int nq = 0, nk = 0;                          // Q (per pair job) and k_bar loads issued
+    int nq = 0, nk = 0;                          // Q (per job) and k_bar loads issued
     auto job = [&](int j, uint32_t slots, int passes) -> bool {
       if (n_ch == 0) return true;                // no block ends before the tile's rows: nothing to load
       if (nq >= 1 && !warp_wait(bar(C::B_QE), (nq - 1) & 1, abort_flag)) return false;
@@ -386,7 +390,7 @@ __global__ void __launch_bounds__(kThreads, 1) topp_select_kernel(const __grid_c
     int t = 0;                                   // chunk steps this slot consumed
 
     // ---- fast path ----
-    // Per pair: (0) the largest and smallest S over H_i; with m = max x
+    // Per head: (0) the largest and smallest S over H_i; with m = max x
     // rounded up, u = m - x >= 0 for every block (one fma, exact sign) and the
     // floored key 2^23 + floor(u inv_r) is one fma rounded toward zero, with
     // inv_r = 2^14 / (max - min) in log2 units. (1, 2) two 3-bit digits of the
@@ -397,7 +401,7 @@ __global__ void __launch_bounds__(kThreads, 1) topp_select_kernel(const __grid_c
     // above it dropped. Then the list, ordered by u (ties: id order), is walked
     // from the mass below the window: a block is kept while the mass before it
     // is below tau_p Z. A row whose window holds more than kListCap blocks
-    // flags the pair for the radix path.
+    // flags its pair of heads for the radix path.
     for (int job = 0; job < n_jobs; ++job) {
       const int hh = job * kHeadSlots + slot;
       if (!takes_part(~0u, job, slot)) continue; // warp-uniform: a ragged group leaves the last slots idle
@@ -467,7 +471,7 @@ __global__ void __launch_bounds__(kThreads, 1) topp_select_kernel(const __grid_c
               } else {
                 // Kept (key < lo) and in-or-below-window (key < hi) as bit words
                 // summed in fp32 from saturated indicators (exact: 16 bits a
-                // half); u goes to the group scratch for the window's blocks.
+                // half).
                 const float t_lo = kMagic + lo, t_hi = kMagic + hi;
                 float k0 = 0.f, k1 = 0.f, h0 = 0.f, h1 = 0.f;
 #pragma unroll
