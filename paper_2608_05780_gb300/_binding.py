@@ -356,6 +356,8 @@ def tile_union_to_csr(tile_union, n_vis, tile):
     """Host CSR (row_ptr, col_idx) of a tile union from evisel_topp_mask."""
     words = np.ascontiguousarray(tile_union.cpu().numpy()).view(np.uint32)
     rows = int(sum(-(-int(nv) // int(tile)) for nv in np.asarray(n_vis, dtype=np.int64)))
+    if rows > len(words):
+        raise IndexError(f"the union holds {len(words)} row tiles, n_vis and tile ask for {rows}")
     bits = np.unpackbits(words[:rows].astype("<u4", copy=False).view(np.uint8), axis=1, bitorder="little")
     row, col = np.nonzero(bits)                 # row by row, ascending within a row
     row_ptr = np.zeros(rows + 1, np.int32)
