@@ -16,10 +16,12 @@
 //   warp / 4). Four heads of the group go at a time: S = Q_h k_bar^T in chunks
 //   of 128 blocks (tcgen05, the products of all slots from one k_bar chunk, one
 //   TMEM tile per slot, given back when its last columns are in registers),
-//   recomputed for every pass over the chunks. Bound by the digit passes' FMA
-//   pipe and issue (60% of the issue slots, FMA pipe 50%): with two heads at a
-//   time, two row warps per scheduler, a mask of 65,664 tokens in blocks of 64
-//   took 2.5 ms, with four 2.0. A block's key is
+//   recomputed for every pass over the chunks. Bound by the digit passes: per
+//   logit 4 comparisons, 3 saturated differences, 4 packed fmas and an ex2 on the
+//   ALU, FMA and XU pipes (about 22 clocks of a warp's scheduler, waits 5%). With
+//   two heads at a time, two row warps per scheduler, a mask of 65,664 tokens in
+//   blocks of 64 took 2.5 ms, with four 2.0, with the indicators on two pipes and
+//   two columns per min / max instruction 1.86. A block's key is
 //   q = floor((max - x) 2^14 / (max - min)) over H_i (0 = the largest logit);
 //   blocks are ordered by key, ties by id.
 //   Fast path (every head), four passes:
@@ -171,13 +173,21 @@ __device__ __forceinline__ void fma2_rz(float& d0, float& d1, float a0, float a1
 
 // Cumulative masses of one digit pass: cm[k] += w for every digit top top[k]
 // above the block's floored key f (both offset by 2^23, so top - f is an exact
-// integer and its saturation the indicator), on the FMA pipe only, two sums
-// per packed fma. With Z, the sum of every w rides along with the last top.
+// integer and its saturation the indicator), two sums per packed fma. With Z,
+// the sum of every w rides along with the last top. What bounds a digit pass is
+// the FMA pipe (measured: 1.57 clocks per scalar add or fma of a warp, 2.3 per
+// packed one), so kSetTops of the indicators are comparisons on the ALU pipe (2
+// clocks each): the mask of 65,664 tokens takes 2272 us with 0, 2182 with 2, 2162
+// with 4, 2175 with 6 and 2198 with all 7 of them.
+constexpr int kSetTops = 4;
 template <int N, bool kWithZ = false>
 __device__ __forceinline__ void cum_add(float (&cm)[N], const float (&top)[N], float f, float w, float& z) {
   float ind[N];
 #pragma unroll
-  for (int k = 0; k < N; ++k) asm("sub.sat.f32 %0, %1, %2;" : "=f"(ind[k]) : "f"(top[k]), "f"(f));
+  for (int k = 0; k < N; ++k) {
+    if (k < kSetTops) asm("set.lt.f32.f32 %0, %1, %2;" : "=f"(ind[k]) : "f"(f), "f"(top[k]));
+    else asm("sub.sat.f32 %0, %1, %2;" : "=f"(ind[k]) : "f"(top[k]), "f"(f));
+  }
 #pragma unroll
   for (int k = 0; k + 1 < N; k += 2) fma2_rn(cm[k], cm[k + 1], ind[k], ind[k + 1], w, w, cm[k], cm[k + 1]);
   if constexpr (N % 2 == 1 && kWithZ) {
@@ -439,11 +449,21 @@ __global__ void __launch_bounds__(kThreads, 1) topp_select_kernel(const __grid_c
               if (pass == 0) {
                 float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
                 float mn[4] = {INFINITY, INFINITY, INFINITY, INFINITY};
+                if (__all_sync(0xffffffffu, jn >= 32)) {     // two columns per instruction
 #pragma unroll
-                for (int e = 0; e < 32; ++e) {
-                  if (e < jn) {
-                    mx[e & 3] = fmaxf(mx[e & 3], __uint_as_float(r[e]));
-                    mn[e & 3] = fminf(mn[e & 3], __uint_as_float(r[e]));
+                  for (int e = 0; e < 32; e += 2) {
+                    const float a = __uint_as_float(r[e]), c = __uint_as_float(r[e + 1]);
+                    const int i = (e >> 1) & 3;
+                    asm("max.f32 %0, %0, %1, %2;" : "+f"(mx[i]) : "f"(a), "f"(c));
+                    asm("min.f32 %0, %0, %1, %2;" : "+f"(mn[i]) : "f"(a), "f"(c));
+                  }
+                } else {
+#pragma unroll
+                  for (int e = 0; e < 32; ++e) {
+                    if (e < jn) {
+                      mx[e & 3] = fmaxf(mx[e & 3], __uint_as_float(r[e]));
+                      mn[e & 3] = fminf(mn[e & 3], __uint_as_float(r[e]));
+                    }
                   }
                 }
                 smax = fmaxf(smax, fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])));
