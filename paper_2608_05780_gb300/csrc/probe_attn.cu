@@ -58,6 +58,8 @@ constexpr int kWarpVLoader = 10;   // the V ring
 constexpr int kRows = 128;
 constexpr int NK = 3;                  // stages of the K ring (the V ring has NS; shared memory holds no more)
 constexpr float kRescaleThreshold = 8.0f;   // log2 units
+constexpr int kWatch = 16;              // tiles that take their max first after one that moved
+constexpr float kSharpSum = 4.f;        // row sum of a first tile (its largest P is 1) below which logits count as sharp
 constexpr float kLn2 = 0.69314718055994531f;
 
 template <int TILE, int D, int NS>
@@ -480,7 +482,14 @@ __device__ __forceinline__ void softmax_epilogue(const ProbeLaunch& L, const Wor
     if (it.kv_count > 0) em_next = mask_word(kv_next);
   }
 
-  bool watch = true;          // warp-uniform: take this tile's max before its P
+  // Warp-uniform: tiles to go that take their max before P. A tile formed early
+  // that has to be formed again costs about half a tile more, the early start
+  // gains a twentieth: after a maximum that moved the next kWatch tiles take the
+  // max first, and likewise after a first tile whose row sums say that a few
+  // keys hold the mass (sharp logits, whose maxima keep moving). Watching one
+  // tile only took 3,115 us where the max first everywhere took 2,814 (two videos of 48,000
+  // visual tokens, 96,000 in all, logits of std 16), this rule 2,845.
+  int watch = 1;
   for (int j = 0; j < it.kv_count; ++j) {
     KvTile kv;
     [[maybe_unused]] uint32_t em_bits = 0xffffffffu;
@@ -575,7 +584,7 @@ __device__ __forceinline__ void softmax_epilogue(const ProbeLaunch& L, const Wor
     };
 
     uint32_t ra[2][32], rb[2][32], pk[32];   // S: first and second half of the tile
-    bool max_first = TILE == 64 || watch;    // (a 64-key tile gains nothing from the early half)
+    bool max_first = TILE == 64 || watch > 0;    // (a 64-key tile gains nothing from the early half)
     if (!max_first) {
       // The running max holds for nearly every tile: P of the first half is
       // formed with it while the tile's max is taken, and stands if no row of
@@ -598,7 +607,7 @@ __device__ __forceinline__ void softmax_epilogue(const ProbeLaunch& L, const Wor
       max_first = __any_sync(0xffffffffu, m_tile > m_used + kRescaleThreshold);
     }
     if (max_first) {
-      // The first tile, a row whose max grew by more than 2^8, or the tile after
+      // The first tile, a row whose max grew by more than 2^8, or the tiles after
       // such a one (maxima that move tend to move again): the max first, then
       // the lazy rescale of the row sum and (not on the first tile) of the O
       // accumulator. With two slots S_j was issued after P_{j-1}.V, so that
@@ -615,11 +624,12 @@ __device__ __forceinline__ void softmax_epilogue(const ProbeLaunch& L, const Wor
       }
       const float m_tile = fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3])) * L.scale_log2;
       const bool need = m_tile > m_used + kRescaleThreshold;
-      watch = __any_sync(0xffffffffu, need);
+      const bool moved = __any_sync(0xffffffffu, need);
+      watch = moved ? kWatch : watch - 1;
       const float alpha = need ? ptx::ex2(m_used - m_tile) : 1.f;
       l_sum *= alpha;
       m_used = need ? m_tile : m_used;
-      if (watch && j > 0) {
+      if (moved && j > 0) {
         if (!two && !warp_wait(bar(C::B_VE + (j - 1) % NS), ((j - 1) / NS) & 1, abort_flag)) {
           ok = false;
           break;
@@ -659,6 +669,7 @@ __device__ __forceinline__ void softmax_epilogue(const ProbeLaunch& L, const Wor
     ptx::tmem_wait_st();
     ptx::tc_fence_before();
     ptx::mbar_arrive(bar_pf);
+    if (TILE == 128 && j == 0) watch = __popc(__ballot_sync(0xffffffffu, l_sum < kSharpSum)) >= 8 ? kWatch : 0;
   }
 
   ok = ok && warp_wait(bar(C::B_OF + slot), 0, abort_flag);
