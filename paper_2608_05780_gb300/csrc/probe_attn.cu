@@ -487,8 +487,8 @@ __device__ __forceinline__ void softmax_epilogue(const ProbeLaunch& L, const Wor
   // gains a twentieth: after a maximum that moved the next kWatch tiles take the
   // max first, and likewise after a first tile whose row sums say that a few
   // keys hold the mass (sharp logits, whose maxima keep moving). Watching one
-  // tile only took 3,115 us where the max first everywhere took 2,814 (two videos of 48,000
-  // visual tokens, 96,000 in all, logits of std 16), this rule 2,845.
+  // tile only took 3,115 us where the max first everywhere took 2,814 (two videos
+  // of 48,000 visual tokens, logits of std 16), this rule 2,845; 64 for 16 the same.
   int watch = 1;
   for (int j = 0; j < it.kv_count; ++j) {
     KvTile kv;
