@@ -89,16 +89,19 @@ def test_evidence_overwrites_what_the_maps_held_and_accumulates_on_it(cuda_lib):
 
 @pytest.mark.gpu
 @pytest.mark.parametrize("tile", [64, 128])
-@pytest.mark.parametrize("order", ["rising", "falling", "one_spike"])
+@pytest.mark.parametrize("order", ["rising", "falling", "one_spike", "two_steps"])
 def test_running_max_over_key_tiles(cuda_lib, tile, order):
     """The row maximum moves by 8 log2 units at every key tile, at none after the
-    first, or by 65 in the last visual tile alone: the accumulator is rescaled at
-    each step, at none, or once."""
-    probe = _custom(frames=(64,), n_text=(33,), hq=5, hkv=1, d=128, tile=tile, window=64)
+    first, by 65 in the last visual tile alone, or by 32 at tile 1 and again at tile
+    21: the accumulator is rescaled at each step, at none, once, or twice with
+    more tiles between than the kernel stays careful for."""
+    probe = _custom(frames=(25 * tile // 16,), n_text=(33,), hq=5, hkv=1, d=128, tile=tile, window=64)
     n = int(probe.cu_seqlens[-1])
     step = np.arange(n) // tile
     if order == "one_spike":
         level = np.where(step == int(probe.n_vis[0] - 1) // tile, 4.0, 0.0)
+    elif order == "two_steps":
+        level = np.where(step >= 21, 4.0, np.where(step >= 1, 2.0, 0.0))
     else:
         level = 0.5 * (step if order == "rising" else step.max() - step)
     s = np.where(np.arange(128) % 3 == 0, 1.0, -1.0)
