@@ -300,14 +300,15 @@ int evisel_topp_mask(const evisel_probe_args* args, int32_t block, float tau_p, 
  *   tok[h, m] = sum_i A~_im (visual m), frame[h, t], head[b, h], aqf[t]
  * as evisel_evidence_reduce() defines them (same layouts).
  *   args   as for the evisel_topp_mask() call that ran on `ws` (q, k, videos, N_v,
- *          heads, head_dim, softmax_scale); `block` its block size.
+ *          heads, head_dim, softmax_scale; the sizes are compared by value and
+ *          another description is refused with EVISEL_EINVAL); `block` its block size.
  *   keep   that call's per-row bits (S_i and the own block).
  *   ws     the workspace of that call (its k_bar is read; coarse scratch grows
  *          by about hq * n_text_total * 32 * W * 4 bytes).
  *   accumulate  0: overwrite tok and frame; 1: add (sum over layers); head and
  *          aqf are recomputed from the resulting frame map.
- * Asynchronous on `stream`. Errors: EVISEL_EINVAL, EVISEL_ESTATE (no evisel_topp_mask on ws),
- * EVISEL_ENOMEM, EVISEL_ECUDA. */
+ * Asynchronous on `stream`. Errors: EVISEL_EINVAL, EVISEL_ESTATE (no evisel_topp_mask on ws, or the
+ * last one failed), EVISEL_ENOMEM, EVISEL_ECUDA. */
 int evisel_coarse_evidence(const evisel_probe_args* args, evisel_ws* ws, int32_t block, const uint32_t* keep,
                            float* tok, float* frame, float* head, float* aqf, int accumulate, void* stream);
 

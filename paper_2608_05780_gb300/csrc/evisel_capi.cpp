@@ -432,8 +432,8 @@ struct evisel_ws {
   void* topp_stage = nullptr;
   size_t topp_stage_bytes = 0;
   cudaEvent_t topp_done = nullptr;
-  int topp_block = 0;               // the last evisel_topp_mask on this workspace
-  int topp_n_videos = 0, topp_n_words = 0, topp_n_tok = 0;
+  std::vector<int32_t> topp_key;    // description of the evisel_topp_mask call in topp_buf (empty: none)
+  int topp_n_words = 0, topp_n_tok = 0;
   size_t topp_kbar_off = 0;
   // coarse map scratch: offsets, block affinities and row normalisers of the text rows
   void* coarse_buf = nullptr;
@@ -477,6 +477,17 @@ bool key_matches(const evisel_probe_args* a, const std::vector<int32_t>& key) {
     if (!same(a->mask_col_idx_h, a->mask_row_ptr_h[rows])) return false;
   }
   return left == 0;
+}
+
+// Description of a builder call by value: the layout of its videos, blocks and
+// k_bar rows, which a coarse map on the same workspace reads.
+std::vector<int32_t> topp_key(const evisel_probe_args* a, int32_t block) {
+  std::vector<int32_t> k = {block, a->num_videos, a->tokens_per_frame, a->hq, a->hkv, a->head_dim};
+  if (a->num_videos > 0) {
+    k.insert(k.end(), a->cu_seqlens_h, a->cu_seqlens_h + a->num_videos + 1);
+    k.insert(k.end(), a->n_vis_h, a->n_vis_h + a->num_videos);
+  }
+  return k;
 }
 
 template <typename T>
@@ -945,6 +956,7 @@ int evisel_topp_mask(const evisel_probe_args* a, int32_t block, float tau_p, uin
   const size_t need = meta + kbar_bytes;
   if (!ws->topp_done && cudaEventCreateWithFlags(&ws->topp_done, cudaEventDisableTiming) != cudaSuccess)
     return cuda_fail(cudaGetLastError(), "event");
+  ws->topp_key.clear();                            // from here on the last call's state is overwritten
   cudaEventSynchronize(ws->topp_done);             // the staging buffer may still feed the last upload
   if (need > ws->topp_bytes) {
     cudaStreamSynchronize(ws->last_stream);
@@ -1011,8 +1023,7 @@ int evisel_topp_mask(const evisel_probe_args* a, int32_t block, float tau_p, uin
   e = launch_topp(L, stream);
   if (e != cudaSuccess) return cuda_fail(e, "top-p launch");
   ws->last_stream = stream;
-  ws->topp_block = block;
-  ws->topp_n_videos = a->num_videos;
+  ws->topp_key = topp_key(a, block);
   ws->topp_n_words = n_words;
   ws->topp_n_tok = n_tok;
   ws->topp_kbar_off = meta;
@@ -1024,9 +1035,12 @@ int evisel_coarse_evidence(const evisel_probe_args* a, evisel_ws* ws, int32_t bl
   const NvtxRange nvtx_range("evisel_coarse_evidence");
   g_last_error.clear();
   if (!a || !ws) return fail(EVISEL_EINVAL, "args or workspace is NULL");
-  if (ws->topp_block == 0) return fail(EVISEL_ESTATE, "no evisel_topp_mask has run on this workspace");
-  if (block != ws->topp_block || a->num_videos != ws->topp_n_videos ||
-      (a->num_videos > 0 && a->cu_seqlens_h[a->num_videos] != ws->topp_n_tok))
+  if (ws->topp_key.empty()) return fail(EVISEL_ESTATE, "no evisel_topp_mask has run on this workspace");
+  if (a->num_videos < 0 || (a->num_videos > 0 && (!a->cu_seqlens_h || !a->n_vis_h)))
+    return fail(EVISEL_EINVAL, "num_videos / cu_seqlens_h / n_vis_h");
+  // The builder's upload and k_bar are read: every size of this call, its
+  // scratch and its grids must be the builder's, which has checked them.
+  if (topp_key(a, block) != ws->topp_key)
     return fail(EVISEL_EINVAL, "args / block do not match the evisel_topp_mask call on this workspace");
   if (a->num_videos == 0) return EVISEL_OK;
   const int npf = a->tokens_per_frame;
