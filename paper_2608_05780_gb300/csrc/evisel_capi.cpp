@@ -654,6 +654,7 @@ int evisel_probe_attention(const evisel_probe_args* args, void* stream_ptr, evis
   cudaGetDevice(&dev);
   if (dev != ws->device) return fail(EVISEL_EINVAL, "workspace belongs to another device");
 
+  ws->probed = false;               // until every launch of this call is out
   if (!planned) {
     std::vector<int32_t> key = plan_key(args);
     ws->plan = Plan();
@@ -725,7 +726,6 @@ int evisel_probe_attention(const evisel_probe_args* args, void* stream_ptr, evis
       if (e != cudaSuccess) return cuda_fail(e, "attn_combine launch");
     }
   }
-  ws->probed = true;
   ws->probe_keep = args->keep != nullptr;
   ws->lse = args->lse;
   ws->q = args->q;
@@ -736,7 +736,11 @@ int evisel_probe_attention(const evisel_probe_args* args, void* stream_ptr, evis
   ws->hq = args->hq;
   ws->tokens_per_frame = args->tokens_per_frame;
   ws->last_stream = stream;
-  if (!P.text_late) return launch_text_sums(ws, ws->d_ev_tok, ws->d_ev_frame, 0, args, stream);
+  if (!P.text_late) {
+    rc = launch_text_sums(ws, ws->d_ev_tok, ws->d_ev_frame, 0, args, stream);
+    if (rc != EVISEL_OK) return rc;
+  }
+  ws->probed = true;
   return EVISEL_OK;
 }
 

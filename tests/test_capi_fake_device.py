@@ -86,3 +86,41 @@ def test_coarse_map_is_refused_after_a_builder_call_that_failed(fake, name):
     assert fake.fake_calls(b"coarse") == n
     assert _topp(fake, ws, built) == 0 and _coarse(fake, ws, built) == 0
     fake.evisel_free(ws)
+
+
+@pytest.mark.parametrize("text_evidence", [0, 1])
+@pytest.mark.parametrize("name,after", [
+    (b"probe_attn", 0), (b"attn_combine", 0), (b"text_evidence", 0), (b"encode", 0), (b"encode", 3), (b"encode", 4),
+    (b"encode", 5)])
+def test_no_evidence_after_a_probe_that_failed(fake, name, after, text_evidence):
+    """A probe call that fails at any of its launches or descriptors leaves
+    nothing to hand out, neither its own half nor an older call's sums, whether
+    it ran on the plan at hand or on a new one."""
+    def probe(ws, args):
+        args.text_evidence = text_evidence
+        return fake.evisel_probe_attention(ctypes.byref(args), None, ctypes.byref(ws))
+
+    def reduce(ws):
+        return fake.evisel_evidence_reduce(ws, MAP, MAP, MAP, MAP, 0, None)
+
+    late = text_evidence and (name == b"text_evidence" or after >= 4)   # then the evidence call's own
+    # 128 key tiles and two text tiles: split kv ranges, so the combine runs too
+    n = 128 * 64
+    row_ptr, cols = np.arange(129), np.arange(128)
+    built, keep0 = _args(cu=[0, n + 100], n_vis=[n], row_ptr=row_ptr, col_idx=list(cols))
+    other, keep1 = _args(cu=[0, n + 99], n_vis=[n], row_ptr=row_ptr, col_idx=list(cols))
+    for args in (built, other):
+        ws = ctypes.c_void_p(None)
+        assert probe(ws, built) == 0 and reduce(ws) == 0
+        fake.fake_fail(name, after)
+        if late:
+            assert probe(ws, args) == 0
+            fake.fake_fail(name, max(after - 4, 0))
+            assert reduce(ws) == ECUDA and reduce(ws) == 0
+        else:
+            assert probe(ws, args) == ECUDA
+            runs = fake.fake_calls(b"evidence")
+            assert reduce(ws) == ESTATE
+            assert fake.fake_calls(b"evidence") == runs
+            assert probe(ws, args) == 0 and reduce(ws) == 0
+        fake.evisel_free(ws)
