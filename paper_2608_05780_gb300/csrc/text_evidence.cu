@@ -419,31 +419,45 @@ __global__ void __launch_bounds__(kThreads, 1) text_evidence_kernel(const __grid
             ptx::tc_fence_after();
             const int valid = min(x.tile_rows, x.n_text - tt * x.tile_rows);   // columns past them add 0
             const float* lrow = lse_s + (grp * nblk + kblk) * L.text_cols;
-            // Blocks of 32 columns; the last may read up to 16 columns past
-            // tile_rows, whose LSE entries are -inf: they are masked below.
+            auto add4 = [&](const uint32_t* r, const float4& nl, int e) {
+              float x0, x1, x2, x3;
+              ptx::unf2(ptx::fma2(ptx::f2(__uint_as_float(r[0]), __uint_as_float(r[1])), scale2, ptx::f2(nl.x, nl.y)),
+                        x0, x1);
+              ptx::unf2(ptx::fma2(ptx::f2(__uint_as_float(r[2]), __uint_as_float(r[3])), scale2, ptx::f2(nl.z, nl.w)),
+                        x2, x3);
+              a2[(2 * e) & 3] = ptx::add2(a2[(2 * e) & 3], ptx::f2(ptx::ex2(x0), ptx::ex2(x1)));
+              a2[(2 * e + 1) & 3] = ptx::add2(a2[(2 * e + 1) & 3], ptx::f2(ptx::ex2(x2), ptx::ex2(x3)));
+            };
+            int c0 = 0;
 #pragma unroll 1
-            for (int c0 = 0; c0 < valid; c0 += 32) {
+            for (; c0 + 32 <= valid; c0 += 32) {
               float4 l4[8];                        // read before the TMEM wait, which covers their latency
               uint32_t r[32];
               ptx::tmem_ld32(tbase + grp * L.text_cols + c0, r);
 #pragma unroll
               for (int e = 0; e < 8; ++e) l4[e] = reinterpret_cast<const float4*>(lrow + c0)[e];
               ptx::tmem_wait_ld();
-              if (c0 + 32 > x.tile_rows) {         // columns no MMA of this step wrote
 #pragma unroll
-                for (int e = 16; e < 32; ++e) r[e] = 0u;
+              for (int e = 0; e < 8; ++e) add4(r + 4 * e, l4[e], e);
+            }
+            // The last columns by 16: past the video's text rows they are the next
+            // video's queries, which may be non-finite, so that their -inf LSE
+            // entries alone would not keep them out of the sums.
+#pragma unroll 1
+            for (; c0 < valid; c0 += 16) {
+              float4 l4[4];
+              uint32_t r[16];
+              ptx::tmem_ld16(tbase + grp * L.text_cols + c0, r);
+#pragma unroll
+              for (int e = 0; e < 4; ++e) l4[e] = reinterpret_cast<const float4*>(lrow + c0)[e];
+              ptx::tmem_wait_ld();
+              if (c0 + 16 > valid) {
+#pragma unroll
+                for (int e = 1; e < 16; ++e)
+                  if (c0 + e >= valid) r[e] = 0u;
               }
 #pragma unroll
-              for (int e = 0; e < 8; ++e) {
-                const float4 nl = l4[e];
-                float x0, x1, x2, x3;
-                ptx::unf2(ptx::fma2(ptx::f2(__uint_as_float(r[4 * e]), __uint_as_float(r[4 * e + 1])), scale2,
-                                    ptx::f2(nl.x, nl.y)), x0, x1);
-                ptx::unf2(ptx::fma2(ptx::f2(__uint_as_float(r[4 * e + 2]), __uint_as_float(r[4 * e + 3])), scale2,
-                                    ptx::f2(nl.z, nl.w)), x2, x3);
-                a2[(2 * e) & 3] = ptx::add2(a2[(2 * e) & 3], ptx::f2(ptx::ex2(x0), ptx::ex2(x1)));
-                a2[(2 * e + 1) & 3] = ptx::add2(a2[(2 * e + 1) & 3], ptx::f2(ptx::ex2(x2), ptx::ex2(x3)));
-              }
+              for (int e = 0; e < 4; ++e) add4(r + 4 * e, l4[e], e);
             }
             ptx::tc_fence_before();
           }

@@ -58,6 +58,31 @@ def test_text_sums_at_row_tile_edges(cuda_lib, n_text, tile, d, hq, hkv):
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("value", [float("nan"), float("inf")])
+@pytest.mark.parametrize("n_text", [1, 37, 129, 250])
+@pytest.mark.parametrize("tile,d,hq,hkv", [(64, 64, 6, 2), (128, 128, 7, 1)])
+def test_non_finite_queries_of_the_next_video_stay_there(cuda_lib, n_text, tile, d, hq, hkv, value):
+    """A text tile is rounded up to 16 rows, which are the next video's first
+    visual rows: their logits must not enter this video's sums. Its maps are those
+    of the call with finite inputs, bit for bit."""
+    import torch
+    probe = _custom(frames=(9, 5), n_text=(n_text, 20), hq=hq, hkv=hkv, d=d, tile=tile, window=2)
+    cut, cols = int(probe.cu_seqlens[1]), int(probe.n_vis[0])
+    qkv = to_device(probe)
+    bad = qkv[0].clone()
+    bad[cut:] = value
+    for te in (False, True):
+        out, ws = run_cuda(cuda_lib, probe, qkv=qkv, text_evidence=te)
+        ws.free()
+        got, ws = run_cuda(cuda_lib, probe, qkv=(bad, *qkv[1:]), text_evidence=te)
+        ws.free()
+        frames = cols // 16
+        for name, n in (("tok", cols), ("frame", frames)):
+            assert torch.equal(got[name][:, :n], out[name][:, :n]), (name, te)
+        assert torch.equal(got["head"][0], out["head"][0]) and torch.equal(got["aqf"][:frames], out["aqf"][:frames])
+
+
+@pytest.mark.gpu
 def test_evidence_overwrites_what_the_maps_held_and_accumulates_on_it(cuda_lib):
     """The overwrite and accumulate kernels on ragged sizes: NaN in the maps is
     overwritten; accumulate adds one fp32 rounding per entry."""
