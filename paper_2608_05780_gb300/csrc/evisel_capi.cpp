@@ -609,6 +609,8 @@ int launch_text_sums(evisel_ws* ws, float* tok, float* frame, int accumulate, co
   T.tok = tok;
   T.frame = frame;
   if (args && args->keep) {
+    T.q = args->q;
+    T.k = args->k;
     T.keep = args->keep;
     T.keep_words = args->keep_words;
     T.keep_block = args->keep_block;

@@ -184,6 +184,8 @@ struct TextEvidenceLaunch {
   float* frame;                     // [hq, total_frames]
   const uint32_t* keep;             // per-row block masks of the probe (as in ProbeLaunch) or null
   int keep_words, keep_block;
+  const void* q;                    // bf16 [N, hq, d] and [N, hkv, d], read with keep only
+  const void* k;
   int* status;
   int max_text;                     // most text rows of a video
   int head_split, text_cols;        // parts of a KV group's heads, text rows per step (set by the launcher)

@@ -202,6 +202,57 @@ def test_topp_chain_at_edges(cuda_lib, name):
     ws.free()
 
 
+@pytest.mark.gpu
+@pytest.mark.parametrize("value", [float("nan"), float("inf")])
+@pytest.mark.parametrize("name", ["group5_b16_d64_t64", "group9_b32_d128_t128"])
+def test_non_finite_keys_that_no_text_row_keeps_add_nothing(cuda_lib, name, value):
+    """After a masked probe a block that no text row keeps adds 0 to the maps
+    whatever its keys hold: the maps are those of finite keys, bit for bit. A
+    non-finite text query likewise adds nothing to the blocks its row drops, where
+    other rows' sums stand."""
+    import torch
+    kw, block = TOPP[name]
+    probe = _custom(**kw)
+    cfg, cu, n_vis = probe.cfg, probe.cu_seqlens, probe.n_vis
+    q, k, v = to_device(probe)
+    keep, uni, ws = cuda_lib.evisel_topp_mask(q, k, cu, n_vis, cfg.tokens_per_frame, cfg.tile, block, 0.3)
+    row_ptr, col_idx = B.tile_union_to_csr(uni, n_vis, cfg.tile)
+    nv, end = int(n_vis[0]), int(cu[1])
+    victims = [1, nv // block - 1]               # blocks of the first video, dropped from its text rows
+    for j in victims:
+        keep[:, j >> 5, nv:end] &= ~(1 << (j & 31))
+
+    def maps(keys, q=q):
+        w = cuda_lib.Workspace()
+        cuda_lib.evisel_probe_attention(q, keys, v, cu, n_vis, cfg.tokens_per_frame, cfg.tile, row_ptr, col_idx, ws=w,
+                                        keep=keep, keep_block=block)
+        out = cuda_lib.evisel_evidence_reduce(w, cfg.hq, n_vis, cfg.tokens_per_frame, len(n_vis))
+        torch.cuda.synchronize()
+        assert cuda_lib.evisel_status(w) == 0
+        w.free()
+        return out
+    bad = k.clone()
+    for j in victims:
+        bad[j * block:(j + 1) * block] = value
+    want, got = maps(k), maps(bad)
+    for j in victims:
+        assert (want[0][:, j * block:(j + 1) * block] == 0).all()
+    for a, b in zip(want, got):
+        assert torch.equal(a, b)
+    for j in victims:                            # kept by the second text row alone
+        keep[:, j >> 5, nv + 1] |= 1 << (j & 31)
+    bad = q.clone()
+    bad[nv] = value
+    want, got = maps(k)[0], maps(k, bad)[0]
+    # one pair per key, its logit summed over d in another order: 2 d 2^-24 sum |q k| scale
+    # below 2 * 128 * 2^-24 * 400 / sqrt(64) = 8e-4 (sum |q k| < 400 asserted)
+    assert (q[nv + 1].float().norm(dim=-1).max() * k[:nv].float().norm(dim=-1).max()).item() < 400
+    for j in victims:
+        a, b = (m[:, j * block:(j + 1) * block] for m in (want, got))
+        assert (a > 0).all() and ((b - a).abs() <= 8e-4 * a).all()
+    ws.free()
+
+
 # --- plans --------------------------------------------------------------------
 
 @pytest.mark.gpu
