@@ -80,19 +80,19 @@ __global__ void __launch_bounds__(256) coarse_logits_kernel(const __grid_constan
   __shared__ __align__(16) float q_s[kLogitRows][D];
   const int h = blockIdx.z;
   int v, grp;
-  if (!row_group(L, blockIdx.y, kLogitRows, v, grp)) return;   // CTA-uniform
+  if (!row_group(L, blockIdx.x, kLogitRows, v, grp)) return;   // CTA-uniform
   const ToppVideo vid = L.vids[v];
   const int row0 = grp * kLogitRows, nr = min(kLogitRows, vid.n_text - row0);
   const int B = L.block, nvb = vid.n_vis / B;
   const int nh = nvb + (row0 + nr - 1) / B;      // blocks that end before the group's last row
-  if (static_cast<int>(blockIdx.x) * kLogitBlocks >= nh) return;
+  if (static_cast<int>(blockIdx.y) * kLogitBlocks >= nh) return;
   const __nv_bfloat16* q = static_cast<const __nv_bfloat16*>(L.q);
   for (int i = threadIdx.x; i < kLogitRows * D; i += blockDim.x) {
     const int r = i / D, e = i % D;
     q_s[r][e] = r < nr ? __bfloat162float(q[(static_cast<int64_t>(vid.start + vid.n_vis + row0 + r) * L.hq + h) * D + e]) : 0.f;
   }
   __syncthreads();
-  const int j = blockIdx.x * kLogitBlocks + threadIdx.x;
+  const int j = blockIdx.y * kLogitBlocks + threadIdx.x;
   if (j >= nh) return;
   const int g = h / (L.hq / L.hkv);
   const uint4* kb = reinterpret_cast<const uint4*>(static_cast<const __nv_bfloat16*>(L.kbar) +
@@ -295,8 +295,9 @@ __global__ void __launch_bounds__(kFinalWarps * 32) coarse_finalize_kernel(const
 template <int D>
 cudaError_t launch_rows(const CoarseLaunch& L, cudaStream_t stream) {
   // Row groups per video: at most total / size full ones and a partial one per
-  // video; CTAs past the last group return at once.
-  dim3 g1((L.max_blocks + kLogitBlocks - 1) / kLogitBlocks, L.total_text / kLogitRows + L.n_videos, L.hq);
+  // video; CTAs past the last group return at once. The groups take grid x: y and
+  // z end at 65,535.
+  dim3 g1(L.total_text / kLogitRows + L.n_videos, (L.max_blocks + kLogitBlocks - 1) / kLogitBlocks, L.hq);
   coarse_logits_kernel<D><<<g1, 256, 0, stream>>>(L);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;

@@ -253,6 +253,32 @@ def test_non_finite_keys_that_no_text_row_keeps_add_nothing(cuda_lib, name, valu
     ws.free()
 
 
+@pytest.mark.gpu
+def test_coarse_map_takes_a_million_text_rows(cuda_lib):
+    """2,048 videos of one frame and 512 text rows, all alike: 67,584 groups of 16
+    text rows, more than a grid holds in y. Every video's maps are bit for bit
+    those of the call on one of them."""
+    import torch
+    n_text, copies = 512, 2048
+    probe = _custom(frames=(1,), n_text=(n_text,), hq=1, hkv=1, d=64, tile=64, window=2)
+    one = to_device(probe)[:2]
+    n = int(probe.cu_seqlens[-1])
+
+    def maps(videos):
+        q, k = (t.repeat(videos, 1, 1) for t in one)
+        cu, n_vis = np.arange(videos + 1, dtype=np.int32) * n, np.full(videos, n - n_text, np.int32)
+        keep, _, ws = cuda_lib.evisel_topp_mask(q, k, cu, n_vis, 16, 64, 16, 0.9, union=False)
+        out = cuda_lib.evisel_coarse_evidence(q, k, cu, n_vis, 16, 64, 16, keep, ws)
+        torch.cuda.synchronize()
+        assert cuda_lib.evisel_status(ws) == 0
+        ws.free()
+        return out
+    want = maps(1)
+    assert (want[0] > 0).all()
+    for name, a, b in zip(("tok", "frame", "head", "aqf"), want, maps(copies)):
+        assert torch.equal(b, a.repeat(copies, 1) if name == "head" else a.repeat(*[1] * (a.dim() - 1), copies)), name
+
+
 # --- plans --------------------------------------------------------------------
 
 @pytest.mark.gpu
