@@ -58,18 +58,26 @@ __device__ __forceinline__ void merge_mz(float& m, float& z, float m2, float z2)
   m = mm;
 }
 
-// The text rows in groups of `per` per video, videos back to back: the video
-// and group of global index i (false past the last group).
-__device__ __forceinline__ bool row_group(const CoarseLaunch& L, int i, int per, int& v, int& grp) {
-  for (v = 0; v < L.n_videos; ++v) {
-    const int n = (L.vids[v].n_text + per - 1) / per;
-    if (i < n) {
-      grp = i;
-      return true;
-    }
-    i -= n;
+// The video and group of the i-th group of `per` things (text rows, visual
+// blocks), where off(v) is the number of things before video v. Video v's groups
+// start at off(v) / per + v: room for a partial group per video, and found by
+// bisection (a linear search in every CTA took most of the call from some
+// hundred videos on). Groups past a video's last thing are empty.
+template <typename Off>
+__device__ __forceinline__ int video_of_group(const CoarseLaunch& L, int i, int per, Off off, int& grp) {
+  int lo = 0, hi = L.n_videos - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (off(L.vids[mid]) / per + mid <= i) lo = mid; else hi = mid - 1;
   }
-  return false;
+  grp = i - (off(L.vids[lo]) / per + lo);
+  return lo;
+}
+
+// The video and group of the i-th group of `per` text rows (false: an empty one).
+__device__ __forceinline__ bool row_group(const CoarseLaunch& L, int i, int per, int& v, int& grp) {
+  v = video_of_group(L, i, per, [](const ToppVideo& x) { return x.text_off; }, grp);
+  return grp * per < L.vids[v].n_text;
 }
 
 constexpr int kLogitRows = 16;                   // text rows per CTA of the logits
@@ -213,15 +221,11 @@ __global__ void __launch_bounds__(kMapWarps * 32) coarse_map_kernel(const __grid
   __shared__ float c_s[32];
   const int h = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int npf = L.tokens_per_frame, B = L.block;
-  int v = 0, chunk = blockIdx.x;                 // chunks of 32 visual blocks, videos back to back
-  for (; v < L.n_videos; ++v) {
-    const int n = (L.vids[v].n_vis / B + 31) / 32;
-    if (chunk < n) break;
-    chunk -= n;
-  }
-  if (v >= L.n_videos) return;                   // CTA-uniform
-  const ToppVideo vid = L.vids[v];
+  int chunk;                                     // of 32 visual blocks
+  const ToppVideo vid =
+      L.vids[video_of_group(L, blockIdx.x, 32, [B](const ToppVideo& x) { return x.vis_off / B; }, chunk)];
   const int j0 = chunk * 32, nb = min(32, vid.n_vis / B - j0);
+  if (nb <= 0) return;                           // CTA-uniform: an empty group
   const int64_t r0 = static_cast<int64_t>(h) * L.total_text + vid.text_off;
   const float* gcol = L.gbuf + r0 * L.pitch + j0 + lane;
   const uint32_t* keep = L.keep + (static_cast<int64_t>(h) * L.n_words + chunk) * L.n_tok + vid.start + vid.n_vis;
@@ -279,9 +283,12 @@ __global__ void __launch_bounds__(kFinalWarps * 32) coarse_finalize_kernel(const
   }
   const int t = (blockIdx.x - L.n_videos * head_blocks) * blockDim.x + threadIdx.x;
   if (t >= L.total_frames) return;
-  int v = 0;                                     // the video that owns frame t
-  while (v + 1 < L.n_videos && L.vids[v + 1].vis_off / npf <= t) ++v;
-  const int n_text = L.vids[v].n_text;
+  int lo = 0, hi = L.n_videos - 1;               // the video that owns frame t
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (L.vids[mid].vis_off / npf <= t) lo = mid; else hi = mid - 1;
+  }
+  const int n_text = L.vids[lo].n_text;
   float s0 = 0.f, s1 = 0.f;
 #pragma unroll 4
   for (int h = 0; h + 1 < L.hq; h += 2) {

@@ -279,6 +279,41 @@ def test_coarse_map_takes_a_million_text_rows(cuda_lib):
         assert torch.equal(b, a.repeat(copies, 1) if name == "head" else a.repeat(*[1] * (a.dim() - 1), copies)), name
 
 
+@pytest.mark.gpu
+def test_coarse_map_finds_every_videos_rows_and_blocks(cuda_lib):
+    """300 videos with 0 to 40 blocks and 0 to 40 text rows: groups of 32 blocks
+    and of 8 and 16 rows, partial and empty ones among them, each found by
+    bisection. Every video's maps are bit for bit those of a call on it alone."""
+    import torch
+    rng = np.random.default_rng(5)
+    frames, text = rng.integers(0, 41, 300), rng.integers(0, 41, 300)
+    frames[[0, 7, 8, 299]] = text[[0, 8, 9, 299]] = 0
+    frames[20], text[20] = 70, 129               # more than one group of each
+    n_vis = (16 * frames).astype(np.int32)
+    cu = np.concatenate([[0], np.cumsum(n_vis + text)]).astype(np.int32)
+    g = torch.Generator(device="cuda").manual_seed(6)
+    q, k = (torch.randn(int(cu[-1]), h, 64, device="cuda", generator=g).bfloat16() for h in (4, 2))
+
+    def maps(q, k, cu, n_vis):
+        keep, _, ws = cuda_lib.evisel_topp_mask(q, k, cu, n_vis, 16, 64, 16, 0.9, union=False)
+        out = cuda_lib.evisel_coarse_evidence(q, k, cu, n_vis, 16, 64, 16, keep, ws)
+        torch.cuda.synchronize()
+        assert cuda_lib.evisel_status(ws) == 0
+        ws.free()
+        return out
+    tok, frame, head, aqf = maps(q, k, cu, n_vis)
+    vis, fr = np.concatenate([[0], np.cumsum(n_vis)]), np.concatenate([[0], np.cumsum(frames)])
+    for b in [0, 1, 6, 7, 8, 9, 10, 19, 20, 21, 298, 299, *range(30, 290, 13)]:
+        if cu[b] == cu[b + 1]:
+            assert (head[b] == 0).all()
+            continue
+        a, e = int(cu[b]), int(cu[b + 1])
+        one = maps(q[a:e].contiguous(), k[a:e].contiguous(), np.array([0, e - a], np.int32), n_vis[b:b + 1])
+        got = (tok[:, vis[b]:vis[b + 1]], frame[:, fr[b]:fr[b + 1]], head[b:b + 1], aqf[fr[b]:fr[b + 1]])
+        for x, y in zip(one, got):
+            assert torch.equal(x, y), b
+
+
 # --- plans --------------------------------------------------------------------
 
 @pytest.mark.gpu
