@@ -217,7 +217,7 @@ def evisel_evidence_reduce(ws, hq, n_vis, tokens_per_frame, num_videos, tok=None
     lib = load()
     if tok is None or frame is None or head is None or aqf is None:
         # The call overwrites every entry unless it accumulates (head and A_qf always).
-        total_vis = sum(map(int, n_vis))
+        total_vis = int(np.sum(n_vis))
         total_frames = total_vis // int(tokens_per_frame)
         new = torch.zeros if accumulate else torch.empty
         if tok is None:

@@ -176,3 +176,19 @@ def test_coarse_evidence_without_workspace(lib):
     a, keep = _args()
     fake = ctypes.c_void_p(FAKE)
     assert lib.evisel_coarse_evidence(ctypes.byref(a), None, 16, fake, fake, fake, fake, fake, 0, None) == -1
+
+
+class _Lib:
+    """Accepts every call; the binding's own work is what runs."""
+    def __getattr__(self, name):
+        return lambda *a: 0
+
+
+@pytest.mark.parametrize("n_vis", [
+    64, np.int32(64), [64], (32, 32), np.array([32, 32], np.int32), np.array([[32], [32]]), np.array(64)])
+def test_maps_to_allocate_take_any_n_vis_that_sums(monkeypatch, n_vis):
+    """Map sizes from a plain number, a sequence or an array of any shape."""
+    monkeypatch.setattr(B, "load", _Lib)
+    stream = type("S", (), {"cuda_stream": 0})()
+    tok, frame, head, aqf = B.evisel_evidence_reduce(B.Workspace(), 4, n_vis, 16, 2, stream=stream, device="cpu")
+    assert tok.shape == (4, 64) and frame.shape == (4, 4) and head.shape == (2, 4) and aqf.shape == (4,)
