@@ -166,13 +166,18 @@ def make_args(q, k, v, cu_seqlens, n_vis, tokens_per_frame, tile, row_ptr, col_i
     nv, nv_p = _i32(n_vis)
     rp, rp_p = _i32(row_ptr)
     ci, ci_p = _i32(col_idx if len(col_idx) else np.zeros(1, np.int32))
-    _, hq, d = q.shape
-    a = ProbeArgs.from_buffer_copy(_PACK.pack(
-        len(nv), cu_p, nv_p, int(tokens_per_frame), int(hq), int(k.shape[1]), int(d), int(tile),
+    fields = (
+        len(nv), cu_p, nv_p, int(tokens_per_frame), int(q.shape[1]), int(k.shape[1]), int(q.shape[2]), int(tile),
         ctypes.c_float(softmax_scale).value,
         q.data_ptr(), k.data_ptr(), v.data_ptr(), rp_p, ci_p, o.data_ptr(), lse.data_ptr(), int(bool(cross_frame)),
         int(bool(text_evidence)), 0 if keep is None else keep.data_ptr(), 0 if keep is None else int(keep.shape[1]),
-        0 if keep is None else int(keep_block)))
+        0 if keep is None else int(keep_block))
+    try:
+        packed = _PACK.pack(*fields)
+    except struct.error:                        # a number past 32 bits: wrapped, for the library to refuse
+        packed = _PACK.pack(*(ctypes.c_int32(x).value if t is ctypes.c_int32 else x
+                              for x, (_, t) in zip(fields, ProbeArgs._fields_)))
+    a = ProbeArgs.from_buffer_copy(packed)
     return a, (cu, nv, rp, ci)
 
 

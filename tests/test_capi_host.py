@@ -192,3 +192,19 @@ def test_maps_to_allocate_take_any_n_vis_that_sums(monkeypatch, n_vis):
     stream = type("S", (), {"cuda_stream": 0})()
     tok, frame, head, aqf = B.evisel_evidence_reduce(B.Workspace(), 4, n_vis, 16, 2, stream=stream, device="cpu")
     assert tok.shape == (4, 64) and frame.shape == (4, 4) and head.shape == (2, 4) and aqf.shape == (4,)
+
+
+def test_arguments_are_packed_as_fields_are_assigned():
+    """One pack fills the struct as ctypes field by field does: dims by index,
+    numbers past 32 bits wrapped (and then refused by the library, not here)."""
+    import torch
+    q, k = torch.zeros(6, 4, 8, 1), torch.zeros(6, 2, 8, 1)
+    o = torch.zeros(1)
+    a, keep = B.make_args(q, k, k, [0, 6], [4], (1 << 32) + 2, -1, [0], [], o, o, softmax_scale=1e300, keep=q,
+                          keep_block=1 << 31)
+    want = B.ProbeArgs()
+    want.tokens_per_frame, want.tile, want.keep_block, want.softmax_scale = (1 << 32) + 2, -1, 1 << 31, 1e300
+    for f in ("tokens_per_frame", "tile", "keep_block", "softmax_scale"):
+        assert getattr(a, f) == getattr(want, f), f
+    assert (a.num_videos, a.hq, a.hkv, a.head_dim, a.keep_words) == (1, 4, 2, 8, 4)
+    assert a.q == a.keep == q.data_ptr() and a.k == a.v == k.data_ptr() and a.o == a.lse == o.data_ptr()
