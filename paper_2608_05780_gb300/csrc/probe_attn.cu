@@ -768,37 +768,42 @@ __global__ void __launch_bounds__(kThreads<TILE>, 1) probe_attn_kernel(const __g
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const uint32_t sbase = ptx::smem_addr(smem);
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + C::OFF_MISC);
+  volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(smem + C::OFF_MISC);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + C::OFF_MISC + 4);
   const int warp = threadIdx.x >> 5;
   const WorkItem it = L.items[blockIdx.x];
 
   if (threadIdx.x == kWarpProducer * 32) setup_and_first_loads<TILE, D, NS>(L, it, sbase, abort_flag);
   if (warp == 0) {
-    ptx::tmem_alloc<C::TMEM_COLS>(ptx::smem_addr(tmem_slot));
+    ptx::tmem_alloc<C::TMEM_COLS>(sbase + C::OFF_MISC);
     ptx::tmem_relinquish();
   }
   ptx::tc_fence_before();
   __syncthreads();
   ptx::tc_fence_after();
-  const uint32_t tmem = *tmem_slot;
 
-  // 256 x 208 + 128 x 88 = 384 x 168 registers, what the launch holds: the
-  // softmax keeps a whole row of S and its P.
+  // 256 x 192 + 128 x 120 = 384 x 168 registers, what the launch holds: the
+  // softmax keeps a whole row of S and its P. What is live at the switch stays
+  // under the launch's 168, so the softmax takes its own copies of the item, the
+  // shared-memory base and the TMEM address after it (without them, or with 88
+  // for the other warps, up to 5 registers spill).
   if (warp >= kWarpProducer) {
-    if constexpr (TILE == 128) ptx::setmaxnreg_dec<88>();
+    if constexpr (TILE == 128) ptx::setmaxnreg_dec<120>();
     if (warp == kWarpProducer) producer<TILE, D, NS, false>(L, it, sbase, abort_flag);
     else if (warp == kWarpVLoader) producer<TILE, D, NS, true>(L, it, sbase, abort_flag);
-    else if (warp == kWarpMma) mma_issuer<TILE, D, NS>(L, it, sbase, tmem, abort_flag);
+    else if (warp == kWarpMma) mma_issuer<TILE, D, NS>(L, it, sbase, *tmem_slot, abort_flag);
   } else {
-    if constexpr (TILE == 128) ptx::setmaxnreg_inc<208>();
-    softmax_epilogue<TILE, D, NS, FSW, EMB>(L, it, warp / 4, sbase, tmem, abort_flag);
+    if constexpr (TILE == 128) ptx::setmaxnreg_inc<192>();
+    const WorkItem own = L.items[blockIdx.x];
+    uint32_t own_base = sbase;
+    asm volatile("" : "+r"(own_base));
+    softmax_epilogue<TILE, D, NS, FSW, EMB>(L, own, warp / 4, own_base, *tmem_slot, abort_flag);
   }
   ptx::tc_fence_before();
   __syncthreads();
   if (warp == 0) {
     ptx::tc_fence_after();
-    ptx::tmem_dealloc<C::TMEM_COLS>(tmem);
+    ptx::tmem_dealloc<C::TMEM_COLS>(*tmem_slot);
   }
 }
 
