@@ -59,7 +59,8 @@ constexpr int kRows = 128;
 constexpr int NK = 3;                  // stages of the K ring (the V ring has NS; shared memory holds no more)
 constexpr float kRescaleThreshold = 8.0f;   // log2 units
 constexpr int kWatch = 16;              // tiles that take their max first after one that moved
-constexpr float kSharpSum = 4.f;        // row sum of a first tile (its largest P is 1) below which logits count as sharp
+constexpr float kSharpSum = 4.f;        // row sum of a first tile (its largest P is 1) below which a row counts as sharp
+constexpr int kSharpRows = 8;           // sharp rows of a warp that make it take the max first
 constexpr float kLn2 = 0.69314718055994531f;
 
 template <int TILE, int D, int NS>
@@ -486,9 +487,15 @@ __device__ __forceinline__ void softmax_epilogue(const ProbeLaunch& L, const Wor
   // that has to be formed again costs about half a tile more, the early start
   // gains a twentieth: after a maximum that moved the next kWatch tiles take the
   // max first, and likewise after a first tile whose row sums say that a few
-  // keys hold the mass (sharp logits, whose maxima keep moving). Watching one
-  // tile only took 3,115 us where the max first everywhere took 2,814 (two videos
-  // of 48,000 visual tokens, logits of std 16), this rule 2,845; 64 for 16 the same.
+  // keys hold the mass (sharp logits, whose maxima keep moving): a quarter of the
+  // warp's rows, since one row that moves makes the warp form the tile again.
+  // Watching one tile only took 3,115 us where the max first everywhere took
+  // 2,814 (two videos of 48,000 visual tokens, logits of std 16), this rule 2,845;
+  // 64 for 16 the same. Rows with few keys in the first tile or none (above the
+  // diagonal, past the tile's rows, dropped by the row's mask) count as sharp:
+  // their maxima are still to come. Leaving them out took the sparse layer of
+  // 24,704 tokens from 1,096 to 1,107 us and made nothing else faster by more
+  // than 0.3%.
   int watch = 1;
   for (int j = 0; j < it.kv_count; ++j) {
     KvTile kv;
@@ -669,7 +676,7 @@ __device__ __forceinline__ void softmax_epilogue(const ProbeLaunch& L, const Wor
     ptx::tmem_wait_st();
     ptx::tc_fence_before();
     ptx::mbar_arrive(bar_pf);
-    if (TILE == 128 && j == 0) watch = __popc(__ballot_sync(0xffffffffu, l_sum < kSharpSum)) >= 8 ? kWatch : 0;
+    if (TILE == 128 && j == 0) watch = __popc(__ballot_sync(0xffffffffu, l_sum < kSharpSum)) >= kSharpRows ? kWatch : 0;
   }
 
   ok = ok && warp_wait(bar(C::B_OF + slot), 0, abort_flag);
