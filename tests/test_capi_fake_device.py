@@ -22,7 +22,8 @@ def fake(tmp_path_factory):
     here = os.path.dirname(os.path.abspath(__file__))
     subprocess.run(["g++", "-std=c++17", "-O1", "-fPIC", "-shared", "-DEVISEL_BUILD_ID=\"fake\"", "-I" + INCLUDE,
                     "-I" + CSRC, "-I" + cuda, os.path.join(here, "fake_cuda.cpp"),
-                    os.path.join(CSRC, "evisel_capi.cpp"), "-o", out, "-Wl,-z,defs"], check=True)
+                    os.path.join(CSRC, "evisel_capi.cpp"), "-o", out, "-Wl,-z,defs",
+                    "-Wl,-Bsymbolic"], check=True)   # its own cuda* calls, also where torch has loaded the runtime
     lib = ctypes.CDLL(out)
     lib.evisel_last_error.restype = ctypes.c_char_p
     lib.fake_fail.argtypes = [ctypes.c_char_p, ctypes.c_int]
