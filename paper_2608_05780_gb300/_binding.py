@@ -186,8 +186,9 @@ def evisel_probe_attention(q, k, v, cu_seqlens, n_vis, tokens_per_frame, tile, r
                            text_evidence=False, keep=None, keep_block=0):
     """Block-sparse GQA varlen probe attention. q/k/v: CUDA bf16 [N, H, d].
     ``cross_frame`` also keeps the partials evisel_cross_frame_evidence reads;
-    ``text_evidence`` makes evisel_evidence_reduce recompute the text-row
-    probabilities from q and k instead of spilling the logits; ``keep`` (from
+    ``text_evidence`` leaves the text rows' evidence sums to
+    evisel_evidence_reduce (q, k and lse must live until then) instead of
+    forming them in this call; ``keep`` (from
     evisel_topp_mask, with its ``keep_block``) restricts every row to its
     retained blocks.
 
@@ -256,8 +257,9 @@ def evisel_probe_evidence_noalloc(q, k, v, cu_seqlens, n_vis, tokens_per_frame, 
 
     For callers that cannot let the library call cudaMalloc: every output
     (o, lse and the four maps) is passed in, and the library's scratch is a
-    fixed 64 MiB static device array (problems that need more are rejected;
-    ``text_evidence`` drops the text-row logit spill, the largest part).
+    fixed 64 MiB static device array (larger problems are rejected; without
+    ``text_evidence``, which changes nothing else here, the text rows' logits
+    count towards that limit).
     Returns the device status word when ``wait_status`` (the call then waits
     for the stream), else None.
     """

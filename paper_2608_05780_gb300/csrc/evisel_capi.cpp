@@ -419,7 +419,7 @@ struct evisel_ws {
   bool probed = false;
   const float* lse = nullptr;
   bool probe_keep = false;          // the last probe ran with per-row block masks
-  const void* q = nullptr;          // the probe's q and k (read by the recompute evidence)
+  const void* q = nullptr;          // the probe's q and k (read by the text sums)
   const void* k = nullptr;
   int hkv = 0, head_dim = 0;
   float scale = 0.f;
@@ -435,7 +435,7 @@ struct evisel_ws {
   std::vector<int32_t> topp_key;    // description of the evisel_topp_mask call in topp_buf (empty: none)
   int topp_n_words = 0, topp_n_tok = 0;
   size_t topp_kbar_off = 0;
-  // coarse map scratch: offsets, block affinities and row normalisers of the text rows
+  // coarse map scratch: block affinities and row normalisers of the text rows
   void* coarse_buf = nullptr;
   size_t coarse_bytes = 0;
 };
@@ -697,7 +697,6 @@ int evisel_probe_attention(const evisel_probe_args* args, void* stream_ptr, evis
     L.hkv = args->hkv;
     L.head_dim = args->head_dim;
     L.tile = args->tile;
-    L.scale = scale;
     L.scale_log2 = scale * 1.4426950408889634f;
     if (args->keep) {
       L.keep = args->keep;

@@ -87,7 +87,6 @@ struct ProbeLaunch {
   int n_tok;
   int hq, hkv, head_dim, tile;
   float scale_log2;                 // softmax_scale * log2(e)
-  float scale;                      // softmax_scale
   // Cross-frame partials of the visual rows (null when not requested):
   // [hq, fs_nnz, tile / fs_span, tile] fp32, fs_nnz = kept visual kv tiles
   // (the mask's nonzeros, in mask order), fs_span = min(N_v, 64) keys per

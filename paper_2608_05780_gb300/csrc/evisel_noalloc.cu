@@ -212,12 +212,14 @@ extern "C" int evisel_probe_evidence_noalloc(const evisel_probe_args* args, floa
   const size_t meta_end = off;
   const size_t o_part_o = take(static_cast<size_t>(c.parts) * 128 * args->head_dim * sizeof(float));
   const size_t o_part_ml = take(static_cast<size_t>(c.parts) * 128 * sizeof(float2));
-  take(static_cast<size_t>(c.spill_floats) * sizeof(float));
+  take(static_cast<size_t>(c.spill_floats) * sizeof(float));   // counted, never used (see make_plan)
   if (off > kScratchBytes || meta_end - 256 > kStageBytes) {
-    const std::string msg = "problem needs " + std::to_string(off) + " bytes of scratch (plan " +
-                            std::to_string(meta_end - 256) + " bytes); the static scratch holds " +
-                            std::to_string(kScratchBytes) + " bytes (plan at most " + std::to_string(kStageBytes) +
-                            "); use evisel_probe_attention for larger problems";
+    const std::string msg = "problem counts " + std::to_string(off) + " bytes of scratch (plan " +
+                            std::to_string(meta_end - 256) + " bytes" +
+                            (args->text_evidence ? "" : ", text logits " + std::to_string(c.spill_floats * 4) +
+                                                            " bytes by the documented limit, which text_evidence = 1 lifts") +
+                            "); the static scratch holds " + std::to_string(kScratchBytes) + " bytes (plan at most " +
+                            std::to_string(kStageBytes) + "); use evisel_probe_attention for larger problems";
     return set_last_error(EVISEL_ENOMEM, msg.c_str());
   }
 
@@ -280,7 +282,6 @@ extern "C" int evisel_probe_evidence_noalloc(const evisel_probe_args* args, floa
     L.hkv = args->hkv;
     L.head_dim = args->head_dim;
     L.tile = args->tile;
-    L.scale = scale;
     L.scale_log2 = scale * 1.4426950408889634f;
     e = launch_probe_attn(L, stream);
     if (e == cudaSuccess && c.groups > 0) {

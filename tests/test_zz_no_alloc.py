@@ -21,7 +21,8 @@ from paper_2608_05780_gb300.build import build
 
 
 def test_noalloc_refuses_oversized_problem_before_any_launch():
-    """The 65,664-token probe needs ~1 GB of scratch: refused with ENOMEM, no GPU needed."""
+    """The 65,664-token probe counts ~1 GB (its text logits, by the documented limit):
+    refused with ENOMEM, no GPU needed."""
     build()
     lib = B.load()
     cfg = wl.CONFIGS["long65k"]
