@@ -36,7 +36,7 @@ def to_device(probe):
 
 def run_cuda(ev, probe, ws=None, maps=None, accumulate=False, qkv=None, text_evidence=False):
     """Probe + evidence on the GPU; returns numpy outputs and the workspace.
-    ``text_evidence``: the evidence recomputed from q and k instead of the spill."""
+    ``text_evidence``: the text rows' sums formed in the evidence call instead of the probe call."""
     import torch
     cfg = probe.cfg
     q, k, v = qkv if qkv is not None else to_device(probe)

@@ -112,15 +112,12 @@ def test_evidence_overwrites_what_the_maps_held_and_accumulates_on_it(cuda_lib):
 
 # --- attention ----------------------------------------------------------------
 
-@pytest.mark.gpu
-@pytest.mark.parametrize("tile", [64, 128])
-@pytest.mark.parametrize("order", ["rising", "falling", "one_spike", "two_steps"])
-def test_running_max_over_key_tiles(cuda_lib, tile, order):
-    """The row maximum moves by 8 log2 units at every key tile, at none after the
-    first, by 65 in the last visual tile alone, or by 32 at tile 1 and again at tile
-    21: the accumulator is rescaled at each step, at none, once, or twice with
-    more tiles between than the kernel stays careful for."""
-    probe = _custom(frames=(25 * tile // 16,), n_text=(33,), hq=5, hkv=1, d=128, tile=tile, window=64)
+def _leveled(tile, order, **kw):
+    """A probe whose logits step from key tile to key tile: up or down by 8 log2
+    units at every one, up by 65 in the last visual tile alone, or by 32 at tile 1
+    and again at tile 21."""
+    probe = _custom(**{**dict(frames=(25 * tile // kw.get("npf", 16),), n_text=(33,), hq=5, hkv=1, d=128, tile=tile,
+                              window=64), **kw})
     n = int(probe.cu_seqlens[-1])
     step = np.arange(n) // tile
     if order == "one_spike":
@@ -134,12 +131,72 @@ def test_running_max_over_key_tiles(cuda_lib, tile, order):
     k = (s * level[:, None, None] + 0.0625 * probe.k).astype(np.float32)
     probe.k[:] = (k.view(np.uint32) & np.uint32(0xFFFF0000)).view(np.float32)
     probe.q[:] = s
+    return probe
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("tile", [64, 128])
+@pytest.mark.parametrize("order", ["rising", "falling", "one_spike", "two_steps"])
+def test_running_max_over_key_tiles(cuda_lib, tile, order):
+    """The row maximum moves at every key tile, at none after the first, in the last
+    visual tile alone, or at tile 1 and again at tile 21: the accumulator is
+    rescaled at each step, at none, once, or twice with more tiles between than the
+    kernel stays careful for."""
+    probe = _leveled(tile, order)
     out, ws = run_cuda(cuda_lib, probe)
     ws.free()
     o_ref, lse_ref = oracle.probe(probe.q, probe.k, probe.v, probe.cu_seqlens, probe.n_vis, probe.cfg.tile,
                                   probe.row_ptr, probe.col_idx)
     check_o(np32(out["o"]), o_ref, order)
     check_lse(np32(out["lse"]), lse_ref, order)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("npf", [16, 64])
+@pytest.mark.parametrize("order", ["one_spike", "two_steps"])
+def test_running_max_with_cross_frame_partials(cuda_lib, order, npf):
+    """The first tiles are flat, so P of a later tile's first half is formed on the
+    old maximum, found too small and formed again, its partials stored twice."""
+    from test_gpu_cross_frame import _check, _gpu, _oracle
+    probe = _leveled(128, order, npf=npf)
+    (aff, eff), (want_aff, want_eff) = _gpu(cuda_lib, probe), _oracle(probe)
+    _check(aff, np.concatenate([np.asarray(x).ravel() for x in want_aff]), f"{order} A_ff")
+    _check(eff, np.concatenate([np.asarray(x).ravel() for x in want_eff]), f"{order} E_ff")
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("block", [16, 128])
+@pytest.mark.parametrize("order", ["one_spike", "two_steps"])
+def test_running_max_with_row_masks(cuda_lib, order, block):
+    """As above under per-row masks that drop a third of the blocks, the masks
+    applied again when P is formed again."""
+    import torch
+    from test_gpu_topp import _sets_from_keep
+    probe = _leveled(128, order, npf=max(block, 16))
+    cfg, cu, n_vis = probe.cfg, probe.cu_seqlens, probe.n_vis
+    n, nv = int(cu[-1]), int(n_vis[0])
+    rng = np.random.default_rng(8)
+    pos = np.arange(n)
+    own = np.where(pos < nv, pos // block, nv // block + (pos - nv) // block)
+    blocks = nv // block + -(-(n - nv) // block)
+    words = -(-blocks // 32)
+    bits = rng.random((cfg.hq, words * 32, n)) < 2 / 3
+    ids = np.arange(words * 32)[:, None]
+    bits = (bits & (ids < own)) | (ids == own)
+    bits[:, 0] |= rng.random((cfg.hq, n)) < 0.9      # the first block mostly kept: a flat first tile
+    packed = (bits.reshape(cfg.hq, words, 32, n).astype(np.uint64) << np.arange(32, dtype=np.uint64)[:, None]).sum(2)
+    keep = torch.from_numpy(packed.astype(np.uint32).view(np.int32)).cuda()
+    q, k, v = to_device(probe)
+    o, lse, ws = cuda_lib.evisel_probe_attention(q, k, v, cu, n_vis, cfg.tokens_per_frame, cfg.tile, probe.row_ptr,
+                                                 probe.col_idx, keep=keep, keep_block=block)
+    torch.cuda.synchronize()
+    assert cuda_lib.evisel_status(ws) == 0
+    ws.free()
+    rows = np.unique(np.concatenate([rng.integers(0, n, 60), np.arange(n - 40, n)]))
+    kept = _sets_from_keep(keep, np.arange(n), cu, n_vis, block)
+    o_ref, lse_ref = oracle.probe_rows_topp(probe.q, probe.k, probe.v, cu, n_vis, block, kept, rows)
+    check_o(np32(o)[rows], o_ref, order)
+    check_lse(np32(lse)[:, rows], lse_ref, order)
 
 
 # --- top-p masks, masked text sums, coarse map ---------------------------------
