@@ -11,8 +11,8 @@
 //   A_qf:     sum over heads / (Hq n_text) (one thread per frame)
 // Both are recomputed from the resulting frame map, so that they accumulate
 // over layers exactly as it does. A few MB move: launches and latency are what
-// the call costs (65,664 tokens: 6 us; the pass that read 940 MB of spilled
-// logits back took 171 us).
+// the call costs (65,664 tokens: 9 us; the pass that read 940 MB of spilled
+// logits back took 164 us).
 #include <cstdint>
 #include <cuda_runtime.h>
 

@@ -34,11 +34,12 @@
 // 128), so one wide text tile per head is cheaper than several narrow ones;
 // the waits of a step (about 150 clocks each even when they are over) are
 // hidden only behind other heads' sums, hence the groups.
-// A pair of columns is one packed fma, two ex2 and one packed add. The call
-// with one CTA per (128 keys, KV group), one thread per key and two CTAs per SM
-// took 415 us on the 8-video batch, 108 us on 65,664 tokens, 34 us on 16,512 and
-// 16.4 us on 4,160; this one 339, 79, 29 and 12.4 us. (The LSE warp with one
-// step's loads in flight, serialised by a branch: 397, 91, 43 and 14.5 us.)
+// A pair of columns is one packed fma, two ex2 and one packed add. The evidence
+// call that forms the sums (this kernel and the maps, 28 heads in 4 groups, d =
+// 128) took 419 us on the 8-video batch, 116 on 65,664 tokens, 37 on 16,512 and 19
+// on 4,160 with one CTA per (128 keys, KV group), one thread per key and two CTAs
+// per SM; with this kernel 351, 87, 31 and 16. The LSE warp needs two steps'
+// loads in flight: with one, serialised by a branch, the kernel takes 6 to 40% more.
 // Every (head, key) has one writer and a fixed summation order. Every wait is
 // bounded; on timeout the CTA records EVISEL_ETIMEOUT and drains its copies
 // and MMAs. The key warps never leave their loop early; after a timeout they

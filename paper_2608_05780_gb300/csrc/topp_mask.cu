@@ -18,10 +18,12 @@
 //   TMEM tile per slot, given back when its last columns are in registers),
 //   recomputed for every pass over the chunks. Bound by the digit passes: per
 //   logit 4 comparisons, 3 saturated differences, 4 packed fmas and an ex2 on the
-//   ALU, FMA and XU pipes (about 22 clocks of a warp's scheduler, waits 5%). With
-//   two heads at a time, two row warps per scheduler, a mask of 65,664 tokens in
-//   blocks of 64 took 2.5 ms, with four 2.0, with the indicators on two pipes and
-//   two columns per min / max instruction 1.86. A block's key is
+//   ALU, FMA and XU pipes (about 22 clocks of a warp's scheduler, waits 5%). The
+//   whole call on 65,664 tokens, 28 heads in 4 groups, blocks of 64 (device time;
+//   near-uniform and clustered inputs): two heads at a time, two row warps per
+//   scheduler, 2,853 and 2,680 us; four 2,398 and 2,197; the indicators on two
+//   pipes and two columns per min / max instruction 2,227 and 2,061. Groups of 1
+//   to 9 heads take 0.5 to 1.0 of their time with two heads at a time. A block's key is
 //   q = floor((max - x) 2^14 / (max - min)) over H_i (0 = the largest logit);
 //   blocks are ordered by key, ties by id.
 //   Fast path (every head), four passes:
@@ -177,8 +179,8 @@ __device__ __forceinline__ void fma2_rz(float& d0, float& d1, float a0, float a1
 // the sum of every w rides along with the last top. What bounds a digit pass is
 // the FMA pipe (measured: 1.57 clocks per scalar add or fma of a warp, 2.3 per
 // packed one), so kSetTops of the indicators are comparisons on the ALU pipe (2
-// clocks each): the mask of 65,664 tokens takes 2272 us with 0, 2182 with 2, 2162
-// with 4, 2175 with 6 and 2198 with all 7 of them.
+// clocks each): the call on 65,664 tokens (near-uniform inputs) takes 2,377 us with
+// 0, 2,240 with 2, 2,227 with 4, 2,232 with 6 and 2,257 with all 7 of them.
 constexpr int kSetTops = 4;
 template <int N, bool kWithZ = false>
 __device__ __forceinline__ void cum_add(float (&cm)[N], const float (&top)[N], float f, float w, float& z) {
