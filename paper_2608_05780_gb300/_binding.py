@@ -122,6 +122,14 @@ def _i32(a):
     return a, a.__array_interface__["data"][0]
 
 
+def _total(n):
+    """int(np.sum(n)); a few plain whole numbers, the usual case, without numpy's 4 to 10 us."""
+    few = n.tolist() if type(n) is np.ndarray and n.ndim == 1 and n.size <= 32 else n
+    if type(few) in (list, tuple) and len(few) <= 32 and all(type(x) is int for x in few):
+        return sum(few)
+    return int(np.sum(n))
+
+
 _raw_stream = None      # torch's own lookup of the current stream's handle, where it has one
 
 
@@ -166,8 +174,9 @@ def make_args(q, k, v, cu_seqlens, n_vis, tokens_per_frame, tile, row_ptr, col_i
     nv, nv_p = _i32(n_vis)
     rp, rp_p = _i32(row_ptr)
     ci, ci_p = _i32(col_idx if len(col_idx) else np.zeros(1, np.int32))
+    dims = q.shape
     fields = (
-        len(nv), cu_p, nv_p, int(tokens_per_frame), int(q.shape[1]), int(k.shape[1]), int(q.shape[2]), int(tile),
+        len(nv), cu_p, nv_p, int(tokens_per_frame), int(dims[1]), int(k.shape[1]), int(dims[2]), int(tile),
         ctypes.c_float(softmax_scale).value,
         q.data_ptr(), k.data_ptr(), v.data_ptr(), rp_p, ci_p, o.data_ptr(), lse.data_ptr(), int(bool(cross_frame)),
         int(bool(text_evidence)), 0 if keep is None else keep.data_ptr(), 0 if keep is None else int(keep.shape[1]),
@@ -223,7 +232,7 @@ def evisel_evidence_reduce(ws, hq, n_vis, tokens_per_frame, num_videos, tok=None
     lib = load()
     if tok is None or frame is None or head is None or aqf is None:
         # The call overwrites every entry unless it accumulates (head and A_qf always).
-        total_vis = int(np.sum(n_vis))
+        total_vis = _total(n_vis)
         total_frames = total_vis // int(tokens_per_frame)
         new = torch.zeros if accumulate else torch.empty
         if tok is None:

@@ -185,7 +185,8 @@ class _Lib:
 
 
 @pytest.mark.parametrize("n_vis", [
-    64, np.int32(64), [64], (32, 32), np.array([32, 32], np.int32), np.array([[32], [32]]), np.array(64)])
+    64, np.int32(64), [64], (32, 32), [np.int32(32)] * 2, [32.0, 32.0], [[32], [32]], np.array([32, 32], np.int32),
+    np.full(64, 1), np.array([[32], [32]]), np.array(64)])
 def test_maps_to_allocate_take_any_n_vis_that_sums(monkeypatch, n_vis):
     """Map sizes from a plain number, a sequence or an array of any shape."""
     monkeypatch.setattr(B, "load", _Lib)
