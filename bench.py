@@ -803,7 +803,7 @@ def bench_ours(args, cfg):
                 "roofline": {"bound": "tensor", "achieved": attn_tflops, "peak": peaks["bf16"], "unit": "TFLOP/s",
                              "frac": attn_tflops / peaks["bf16"],
                              "traffic": _traffic(cfg.name),
-                             "kernel": "probe_attn (evisel_probe_attention: probe_attn_kernel + attn_combine)",
+                             "kernel": "probe_attn (evisel_probe_attention: probe_attn_kernel + attn_combine + text_evidence_kernel)",
                              "peak_source": f"{peaks['source']} bf16 burst"},
                 "intra_frame": {"ms": if_ms, "gbs": if_bytes / (if_ms * 1e-3) / 1e9,
                                 "frac_of_hbm": if_bytes / (if_ms * 1e-3) / 1e9 / peaks["hbm"], "bytes": if_bytes,
